@@ -147,9 +147,13 @@ typedef struct {
     int32_t n_steps;          /* slices in the window, 1..12288                  */
     int32_t precision;        /* WAKE_FP64 or WAKE_MIXED                         */
     int32_t flags;            /* WAKE_DUMP_* bits                                */
-    int32_t block_threads;    /* FP64, mobile ions, RK4: threads per wake
+    int32_t block_threads;    /* FP64, mobile ions, RK4: threads per block
                                  (multiple of 32, 64..512); 0 = library
-                                 default (256; 512 with mobile ions or RK4)    */
+                                 default (512 with mobile ions or RK4, 256
+                                 with beam grids).  FP64 without these: 0 =
+                                 the on-chip march (blocks of up to 128
+                                 threads, up to 16 of them by the ring
+                                 count), else one block of that many threads */
     int32_t rings_per_thread; /* MIXED: 2, 4 or 8 rings per thread; 0 = auto  */
     int32_t cluster_ctas;     /* MIXED: CTAs per wake, 1..16 (> 1: a thread-
                                  block cluster); 0 = automatic.  The threads

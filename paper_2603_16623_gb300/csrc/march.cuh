@@ -235,8 +235,9 @@ __device__ __forceinline__ ff acc_add_prod(ff a, float x, float y) { return ff_a
 // barrier, which every block passes only after it read the buffer).
 // ---------------------------------------------------------------------------
 constexpr int kMaxWakeCtas = 8;
+constexpr int kMaxPartCtas = 16;                       // (the FP64 on-chip march's largest cluster)
 constexpr int kPartSlot = 64;                          // bytes per block total
-constexpr int kPartBuf = kMaxWakeCtas * kPartSlot;     // one buffer
+constexpr int kPartBuf = kMaxPartCtas * kPartSlot;     // one buffer
 struct WakeCtas {
     int rank = 0, size = 1;
     unsigned char* part = nullptr;  // 2 x kPartBuf bytes of shared memory (size > 1)

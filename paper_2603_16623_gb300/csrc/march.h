@@ -25,6 +25,15 @@ cudaError_t launch_march_fast(const WakeDev<PrecMixed>* d_wakes, const int32_t* 
 // sized so that the stage never lowers the number of blocks an SM holds
 // (clusters > 1: the cluster march's footprint)
 int32_t march_stage_particles(int32_t threads, int32_t k_rings, int32_t cluster_ctas, int32_t want);
+// the double-precision march of gridless AB2 wakes (march_f64.cuh): the
+// shape of a wake of n rings (a pure function of n), and its launch
+struct F64Shape {
+    int32_t threads, k, cl;
+};
+F64Shape f64_shape(int32_t n);
+cudaError_t launch_march_f64(const WakeDev<PrecF64>* d_wakes, const int32_t* d_order, int32_t n_wakes,
+                             int32_t max_slices, int32_t mode, int32_t threads, int32_t k_rings, int32_t cl,
+                             int32_t n_max, cudaStream_t st);
 // the cluster march: clusters of cl CTAs of `threads` threads, k_rings = 2,
 // 4 or 8 rings per thread
 cudaError_t launch_march_cluster(const WakeDev<PrecMixed>* d_wakes, const int32_t* d_order, int32_t n_wakes,

@@ -668,6 +668,10 @@ wake_status launch_one(wake_handle* h, const WakeDev<P>* d_desc, int32_t max_sli
             else WK_CUDA(launch_march_fast(d_desc, nullptr, 1, max_slices, mode, t, k, stage, h->st));
             return WAKE_OK;
         }
+    } else if (h->fast_threads > 0) {
+        WK_CUDA(launch_march_f64(d_desc, nullptr, 1, max_slices, mode, h->fast_threads, h->fast_k, h->fast_cl, h->n,
+                                 h->st));
+        return WAKE_OK;
     }
     int32_t mb_cap = 0;
     size_t smem = march_smem(h->n, h->n_pad, h->real_bytes(), kMaxSliceParticles, &mb_cap);
@@ -858,6 +862,12 @@ wake_status batch_bucket(const std::vector<wake_handle*>& hs, const FastShape& s
             if (e != cudaSuccess) return fail(WAKE_ECUDA, "batched march launch failed: %s", cudaGetErrorString(e));
             return WAKE_OK;
         }
+    } else if (fast_threads > 0) {
+        e = launch_march_f64(static_cast<const WakeDev<P>*>(d_buf), d_order, n, max_slices, MODE_MARCH, fast_threads,
+                             shape.k, shape.cl, n_max, st);
+        cudaFreeAsync(d_buf, st);
+        if (e != cudaSuccess) return fail(WAKE_ECUDA, "batched march launch failed: %s", cudaGetErrorString(e));
+        return WAKE_OK;
     }
     int32_t mb_cap = 0;
     size_t smem = march_smem(n_max, pad_max, hs[0]->real_bytes(), kMaxSliceParticles, &mb_cap);
@@ -908,6 +918,8 @@ int32_t gm_cluster_for(int32_t positions, int32_t threads, int32_t per_thread) {
 }
 
 double predicted_slice_us(const wake_handle* h) {
+    // FP64 on chip: the scans' chain, then a block's FP64 pipes (rings per thread)
+    if (h->fast_threads > 0 && h->prec == WAKE_FP64) return 17.0 + 8.0 * h->fast_k + 0.25 * h->fast_cl;
     if (h->fast_threads > 0) {
         FastShape f;
         f.threads = h->fast_threads;
@@ -1501,6 +1513,14 @@ wake_status wake_init(const wake_config* cfg, const wake_plasma_desc* plasma, co
             delete h;
             return fs;
         }
+    }
+    // FP64 gridless AB2 wakes: the on-chip double-precision march, unless the
+    // caller asks for one block of a given size (block_threads)
+    if (h->prec == WAKE_FP64 && !ions && !rk4 && !grid && !cfg->block_threads) {
+        const F64Shape f = f64_shape(n);
+        shape.threads = f.threads;
+        shape.k = f.k;
+        shape.cl = f.cl;
     }
     h->fast_threads = shape.threads;
     h->fast_k = shape.k;
