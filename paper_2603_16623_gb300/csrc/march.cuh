@@ -250,6 +250,11 @@ struct WakeCtas {
             __syncthreads();
         }
     }
+    // Before any block stores into another's shared memory: every block of
+    // the cluster has started (a store to a block not yet running faults).
+    __device__ __forceinline__ void start() const {
+        if (size > 1) sync();
+    }
     // this block's value v to slot `rank` of every block's current buffer,
     // then the barrier; returns the buffer (its slots in rank order)
     template <class T>
@@ -506,6 +511,7 @@ march_kernel(const WakeDev<P>* __restrict__ wakes, const int32_t* __restrict__ o
         C.size = (int)c;
         C.part = s_part;
     }
+    C.start();
     const int wi = blockIdx.x / C.size;
     const WakeDev<P>& W = wakes[order ? order[wi] : wi];
     const int T = blockDim.x;

@@ -291,7 +291,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
     for (int i = tid; i < cap; i += blockDim.x) cnt_a[i] = 0;
 
     if (tid < CTL_N) s_ctl[tid] = W.ctl[tid];
-    __syncthreads();
+    cl.sync();  // every CTA has started before any stores into another's shared memory
     // (status and slice are the same for every CTA of the cluster)
     if (s_ctl[CTL_STATUS] != 0) return;
     int slice = s_ctl[CTL_NEXT];

@@ -288,6 +288,7 @@ march_f64_kernel(const WakeDev<PrecF64>* __restrict__ wakes, const int32_t* __re
         C.size = (int)c;
         C.part = s_part;
     }
+    C.start();
     const int wi = blockIdx.x / C.size;
     const WakeDev<PrecF64>& W = wakes[order ? order[wi] : wi];
     const int T = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

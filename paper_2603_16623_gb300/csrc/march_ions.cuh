@@ -131,6 +131,7 @@ march_ions_kernel(const WakeDev<P>* __restrict__ wakes, const int32_t* __restric
         C.size = (int)c;
         C.part = s_part;
     }
+    C.start();
     const int wi = blockIdx.x / C.size;
     const WakeDev<P>& W = wakes[order ? order[wi] : wi];
     const int T = blockDim.x;

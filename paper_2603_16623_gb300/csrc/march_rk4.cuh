@@ -221,6 +221,7 @@ march_rk4_kernel(const WakeDev<P>* __restrict__ wakes, const int32_t* __restrict
         C.size = (int)c;
         C.part = s_part;
     }
+    C.start();
     const int wi = blockIdx.x / C.size;
     const WakeDev<P>& W = wakes[order ? order[wi] : wi];
     const int T = blockDim.x;
