@@ -23,7 +23,7 @@ __device__ __forceinline__ float2 split_ff(double v) {
 template <class R>
 __global__ void ring_init_kernel(const double* __restrict__ edges, const double* __restrict__ cell_density,
                                  int32_t n, int32_t n_total, double density, R* w, R* wh, R* rho, R* rho_lo, R* ur,
-                                 R* frho, R* fur, int32_t* rid, float4* ctab) {
+                                 R* frho, R* fur, int32_t* rid, RingTab ctab) {
     for (int32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n_total; j += gridDim.x * blockDim.x) {
         const int32_t cell = j < n ? j : j - n;
         const double sign = j < n ? 1.0 : -1.0;
@@ -36,14 +36,15 @@ __global__ void ring_init_kernel(const double* __restrict__ edges, const double*
         wh[j] = (R)whj;
         rho[j] = (R)c;
         rho_lo[j] = (R)(c - (double)(R)c);  // mixed path: rho = rho + rho_lo
-        if (ctab) {     // mixed path: per-ring constants, float-float from FP64
+        if (ctab.t) {     // mixed path: per-ring constants, float-float from FP64
             double l0 = log(c);
             float2 a = split_ff(c), b = split_ff(l0), e = split_ff(wj), f = split_ff(whj), g = split_ff(wj * l0);
-            ctab[3 * j] = make_float4(a.x, a.y, b.x, b.y);
-            ctab[3 * j + 1] = make_float4(e.x, e.y, f.x, f.y);
+            float4* t = const_cast<float4*>(ctab.t) + ctab.at(j);
+            t[0] = make_float4(a.x, a.y, b.x, b.y);
+            t[ctab.part] = make_float4(e.x, e.y, f.x, f.y);
             // the spare slots: 1/w and 1/rho0 as the march takes them (the
             // same float reciprocals it would take of the same floats)
-            ctab[3 * j + 2] = make_float4(g.x, g.y, __frcp_rn(e.x), __frcp_rn(a.x));
+            t[2 * ctab.part] = make_float4(g.x, g.y, __frcp_rn(e.x), __frcp_rn(a.x));
         }
         ur[j] = 0;
         frho[j] = 0;
@@ -254,7 +255,7 @@ cudaError_t launch_gather_ctl(const int32_t* const* ctls, int32_t n, int32_t* ou
 template <class R>
 cudaError_t launch_ring_init(const double* edges, const double* cell_density, int32_t n, int32_t n_total,
                              double density, R* w, R* wh, R* rho, R* rho_lo, R* ur, R* frho, R* fur, int32_t* rid,
-                             float4* ctab, cudaStream_t st) {
+                             RingTab ctab, cudaStream_t st) {
     int grid = (n_total + 255) / 256;
     ring_init_kernel<R><<<grid, 256, 0, st>>>(edges, cell_density, n, n_total, density, w, wh, rho, rho_lo, ur,
                                               frho, fur, rid, ctab);
@@ -282,9 +283,9 @@ template cudaError_t launch_march<PrecMixed>(const WakeDev<PrecMixed>*, const in
                                              int32_t, size_t, int32_t, int32_t, cudaStream_t);
 template cudaError_t launch_ring_init<double>(const double*, const double*, int32_t, int32_t, double, double*,
                                               double*, double*, double*, double*, double*, double*, int32_t*,
-                                              float4*, cudaStream_t);
+                                              RingTab, cudaStream_t);
 template cudaError_t launch_ring_init<float>(const double*, const double*, int32_t, int32_t, double, float*, float*,
-                                             float*, float*, float*, float*, float*, int32_t*, float4*,
+                                             float*, float*, float*, float*, float*, int32_t*, RingTab,
                                              cudaStream_t);
 template <class P>
 cudaError_t launch_march_rk4(const WakeDev<P>* d_wakes, const int32_t* d_order, int32_t n_wakes,

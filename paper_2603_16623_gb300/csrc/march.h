@@ -51,7 +51,7 @@ cudaError_t launch_gather_ctl(const int32_t* const* ctls, int32_t n, int32_t* ou
 template <class R>
 cudaError_t launch_ring_init(const double* edges, const double* cell_density, int32_t n, int32_t n_total,
                              double density, R* w, R* wh, R* rho, R* rho_lo, R* ur, R* frho, R* fur, int32_t* rid,
-                             float4* ctab, cudaStream_t st);
+                             RingTab ctab, cudaStream_t st);
 // the march with the RK4 ring integrator (march_rk4.cuh), one block per wake
 // or a thread-block cluster of cluster_ctas (<= 8) blocks per wake
 template <class P>

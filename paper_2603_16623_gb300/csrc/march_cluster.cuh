@@ -269,7 +269,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
     const int p0 = tid * K;                    // local positions [p0, p0 + K)
     const int cap = TK + 8;
     const bool last_cta = crank == csize - 1;  // holds the last ring and region n
-    const float4* __restrict__ ctab = W.ctab;
+    const RingTab ctab = W.ctab;
 
     unsigned char* sscan = smem;
     FastSmem sm;
@@ -608,7 +608,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
             lp[k] = 0.f;
             if (p < nl) {
                 const int a = SW::at(p);
-                RingConst c = ring_const(ctab, idv[k]);
+                RingConst c = ring_const<K>(ctab, idv[k]);
                 const R dl = ff_to_f(ff_acc(ff{rh[k], sm.rl[a]}, ff_neg(c.r0)));
                 lp[k] = log1pf(dl * c.ir0);
                 sw = ff_acc(sw, c.w);
@@ -646,7 +646,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                     lb = staged ? cnt_a[a] : lb + cnt_a[a];
                     cnt_a[a] = 0;  // read for the last time this slice
                 }
-                RingConst c = ring_const(ctab, idv[k]);
+                RingConst c = ring_const<K>(ctab, idv[k]);
                 R r = rh[k], u = ur[k];
                 A rf = {r, sm.rl[a]};
                 A r2 = ff_mul(rf, rf);
@@ -701,13 +701,14 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                 int p = p0 + k;
                 if (p < nl) {
                     const int a = SW::at(p);
-                    const float4 cw = __ldg(ctab + 3 * idv[k] + 1);
+                    const float4* ct = ring_tab<K>(ctab, idv[k]);
+                    const float4 cw = __ldg(ct + ctab.part);
                     const R w = cw.x, wh = cw.z;
                     R r = rh[k], u = ur[k], dpr = dprv[k], ip = IPB(k), iR = IR(k);
                     sm.T[a] = ff_to_f(ff_acc(Ttot, ff_neg(Tacc)));
                     Tacc = ff_add_f(Tacc, tv[k]);
                     R above = ff_to_f(ff_acc(Ttot, ff_neg(Tacc)));
-                    R dpz = -(above + (1.f - wh * __ldg(reinterpret_cast<const float*>(ctab + 3 * idv[k] + 2) + 2)) * tv[k]);
+                    R dpz = -(above + (1.f - wh * __ldg(reinterpret_cast<const float*>(ct + 2 * ctab.part) + 2)) * tv[k]);
                     tv[k] = dpz;
                     R pb = pbv[k];
                     R g = 0.5f * (1.f + u * u + pb * pb) * ip;

@@ -79,8 +79,15 @@ struct RingConst {
     ff r0, ln0, w, wh, wl0;  // rho0, ln rho0, w, what, w ln rho0
     float iw, ir0;           // 1/w and 1/rho0 (of the high parts, rounded to nearest)
 };
-__device__ __forceinline__ RingConst ring_const(const float4* __restrict__ ctab, int id) {
-    float4 a = __ldg(ctab + 3 * id), b = __ldg(ctab + 3 * id + 1), c = __ldg(ctab + 3 * id + 2);
+// (K, the layout's rings per thread, at compile time)
+template <int K>
+__device__ __forceinline__ const float4* ring_tab(const RingTab& tab, int id) {
+    return tab.t + ((id & (K - 1)) * tab.nc + id / K);
+}
+template <int K>
+__device__ __forceinline__ RingConst ring_const(const RingTab& tab, int id) {
+    const float4* t = ring_tab<K>(tab, id);
+    float4 a = __ldg(t), b = __ldg(t + tab.part), c = __ldg(t + 2 * tab.part);
     return {{a.x, a.y}, {a.z, a.w}, {b.x, b.y}, {b.z, b.w}, {c.x, c.y}, c.z, c.w};
 }
 
@@ -403,7 +410,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
     const int p0 = tid * K;
     const int TK = T * K;
     const int cap = TK + 8;
-    const float4* __restrict__ ctab = W.ctab;
+    const RingTab ctab = W.ctab;
 
     unsigned char* sscan = smem;
     FastSmem sm;
@@ -598,7 +605,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
             lp[k] = 0.f;
             if (p < n) {
                 const int a = SW::at(p);
-                RingConst c = ring_const(ctab, idv[k]);
+                RingConst c = ring_const<K>(ctab, idv[k]);
                 const R dl = ff_to_f(ff_acc(ff{rh[k], sm.rl[a]}, ff_neg(c.r0)));  // rho - rho0
                 lp[k] = log1pf(dl * c.ir0);
                 sw = ff_acc(sw, c.w);
@@ -623,7 +630,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
             if (p < n) {
                 const int a = SW::at(p);
                 if (m > 0) lb += t_cnt[a];  // beam particles strictly below ring p
-                RingConst c = ring_const(ctab, idv[k]);
+                RingConst c = ring_const<K>(ctab, idv[k]);
                 R r = rh[k], u = ur[k];
                 A rf = {r, sm.rl[a]};  // rho in float-float
                 A r2 = ff_mul(rf, rf);
@@ -672,13 +679,14 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
                 int p = p0 + k;
                 if (p < n) {
                     const int a = SW::at(p);
-                    const float4 cw = __ldg(ctab + 3 * idv[k] + 1);  // w, what (hi parts)
+                    const float4* ct = ring_tab<K>(ctab, idv[k]);
+                    const float4 cw = __ldg(ct + ctab.part);  // w, what (hi parts)
                     const R w = cw.x, wh = cw.z;
                     R r = rh[k], u = ur[k], dpr = dprv[k], ip = IPB(k), iR = IR(k);
                     sm.T[a] = ff_to_f(ff_acc(Ttot, ff_neg(Tacc)));
                     Tacc = ff_add_f(Tacc, tv[k]);
                     R above = ff_to_f(ff_acc(Ttot, ff_neg(Tacc)));
-                    R dpz = -(above + (1.f - wh * __ldg(reinterpret_cast<const float*>(ctab + 3 * idv[k] + 2) + 2)) * tv[k]);
+                    R dpz = -(above + (1.f - wh * __ldg(reinterpret_cast<const float*>(ct + 2 * ctab.part) + 2)) * tv[k]);
                     tv[k] = dpz;
                     R pb = pbv[k];
                     R g = 0.5f * (1.f + u * u + pb * pb) * ip;

@@ -252,7 +252,7 @@ wake_status prepare_impl(wake_handle* h, cudaStream_t st) {
     WK_CUDA(launch_reset_ctl(h->d_ctl, st));
     WK_CUDA(launch_ring_init<R>(h->d_edges, h->d_density, h->n_ion ? h->n_ion : n, n, h->density, const_cast<R*>(D.w),
                                 const_cast<R*>(D.wh), D.rho[0],
-                                D.rho_lo, D.ur[0], D.frho[0], D.fur[0], D.rid[0], const_cast<float4*>(D.ctab),
+                                D.rho_lo, D.ur[0], D.frho[0], D.fur[0], D.rid[0], D.ctab,
                                 st));
     const size_t rb = h->real_bytes();
     WK_CUDA(cudaMemsetAsync(h->d_boff, 0, ((size_t)ns + 1) * sizeof(int32_t), st));
@@ -351,9 +351,15 @@ wake_status init_impl(wake_handle* h, const wake_config* cfg, const wake_plasma_
     }
     WK_TRY(dalloc_t(h, n, &D.rho_lo));
     if (h->prec == WAKE_MIXED) {  // every mixed march takes its constants from the table
+        // laid out for the rings a thread of this wake's march takes
+        const int32_t per = h->fast_threads ? h->fast_k
+                          : ((h->n_ion ? h->n_ion : n) + h->threads * h->gm_cl - 1) / (h->threads * h->gm_cl);
+        int32_t shift = 0;
+        while (shift < 3 && (1 << shift) < per) ++shift;
+        D.ctab = ring_tab_layout(n, shift);
         float4* ct;
-        WK_TRY(dalloc_t(h, (size_t)3 * n, &ct));
-        D.ctab = ct;
+        WK_TRY(dalloc_t(h, (size_t)3 * D.ctab.part, &ct));
+        D.ctab.t = ct;
     }
     R** scratch[] = {&D.bb, &D.psib, &D.gam, &D.dpr, &D.tt, &D.cA, &D.cB, &D.cC};
     for (R** sp : scratch) WK_TRY(dalloc_t(h, n, sp));
@@ -1123,7 +1129,7 @@ wake_status state_io(wake_handle* h, bool export_, int32_t slice, double* rho, d
         const int b = ctl[CTL_BUF];
         double* outs[4] = {rho, ur, fr, fu};
         if (e == cudaSuccess)
-            e = launch_export_state<R>(D.rid[b], D.rho[b], D.rho_lo, D.ur[b], D.frho[b], D.fur[b], h->n, D.ctab,
+            e = launch_export_state<R>(D.rid[b], D.rho[b], D.rho_lo, D.ur[b], D.frho[b], D.fur[b], h->n, D.ctab.t,
                                        t[0], t[1], t[2], t[3], h->st);
         for (int k = 0; k < 4 && e == cudaSuccess; ++k)
             if (outs[k]) e = cudaMemcpyAsync(outs[k], t[k], bytes, cudaMemcpyDeviceToHost, h->st);
@@ -1132,7 +1138,7 @@ wake_status state_io(wake_handle* h, bool export_, int32_t slice, double* rho, d
         for (int k = 0; k < 4 && e == cudaSuccess; ++k)
             if (ins[k]) e = cudaMemcpyAsync(t[k], ins[k], bytes, cudaMemcpyHostToDevice, h->st);
         if (e == cudaSuccess)
-            e = launch_import_state<R>(t[0], t[1], ifr ? t[2] : nullptr, ifu ? t[3] : nullptr, h->n, D.ctab,
+            e = launch_import_state<R>(t[0], t[1], ifr ? t[2] : nullptr, ifu ? t[3] : nullptr, h->n, D.ctab.t,
                                        D.rho[0], D.rho_lo, D.ur[0], D.frho[0], D.fur[0], D.rid[0], h->d_ctl, slice,
                                        h->st);
     }
