@@ -266,6 +266,24 @@ __device__ __forceinline__ T warp_incl_scan(T v, Op op) {
     return v;
 }
 
+// the same over lanes [0, n) only, the others holding the identity: the
+// steps of n lanes give bitwise what all five would
+template <bool REV, class T, class Op>
+__device__ __forceinline__ T warp_incl_scan_n(T v, Op op, int n) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        if (off >= n) break;
+        T o = REV ? shfl_dn_t(v, off) : shfl_up_t(v, off);
+        bool take = REV ? (lane + off < 32) : (lane >= off);
+        if (take) v = op(o, v);
+    }
+    return v;
+}
+// the lane that holds the fold of lanes [0, n) after warp_incl_scan_n (in
+// the association that the full scan leaves in lane 31)
+__device__ __forceinline__ int scan_last_lane(int n) { return n > 1 ? (1 << (32 - __clz(n - 1))) - 1 : 0; }
+
 template <bool REV, class T, class Op>
 __device__ T block_excl_scan(T v, Op op, T ident, T* sbuf, T& total) {
     const int lane = threadIdx.x & 31;
@@ -401,10 +419,10 @@ __device__ __forceinline__ T block_excl_scan1(T v, Op op, T ident, T* sbuf, T& t
     if (REV ? (lane == 0) : (lane == 31)) sbuf[warp] = inc;
     __syncthreads();
     T wv = lane < nw ? sbuf[lane] : ident;
-    T winc = warp_incl_scan<REV>(wv, op);
+    T winc = warp_incl_scan_n<REV>(wv, op, nw);
     T wex = REV ? shfl_dn_t(winc, 1) : shfl_up_t(winc, 1);
     if (REV ? (lane == 31) : (lane == 0)) wex = ident;
-    total = shfl_idx_t(winc, REV ? 0 : 31);
+    total = shfl_idx_t(winc, REV ? 0 : scan_last_lane(nw));
     return op(shfl_idx_t(wex, warp), lex);
 }
 
@@ -423,44 +441,74 @@ __device__ __forceinline__ Pair<T> block_excl_scan_fwd_rev1(T fx, T ry, T zero, 
     __syncthreads();
     T wx = lane < nw ? sbuf[lane].x : zero;
     T wy = lane < nw ? sbuf[lane].y : zero;
-    T sx = warp_incl_scan<false>(wx, OpAdd());
-    T sy = warp_incl_scan<true>(wy, OpAdd());
+    T sx = warp_incl_scan_n<false>(wx, OpAdd(), nw);
+    T sy = warp_incl_scan_n<true>(wy, OpAdd(), nw);
     T qx = shfl_up_t(sx, 1), qy = shfl_dn_t(sy, 1);
     if (lane == 0) qx = zero;
     if (lane == 31) qy = zero;
-    tx = shfl_idx_t(sx, 31);
+    tx = shfl_idx_t(sx, scan_last_lane(nw));
     ty = shfl_idx_t(sy, 0);
     return {acc_add(shfl_idx_t(qx, warp), ex), acc_add(shfl_idx_t(qy, warp), ey)};
 }
 
-template <bool TOT, class R>
-__device__ __forceinline__ void block_excl_scan_mat_fwd_rev1(Mat2<R> mf, Mat2<R> mr, Pair<Mat2<R>>* sbuf,
-                                                             Mat2<R>& ef, Mat2<R>& er, Mat2<R>& tf, Mat2<R>& tr) {
+// The exclusive sum of t and the exclusive forward and reverse products of
+// mf and mr with one barrier (each as its own one-barrier scan would give
+// it); totals in tt, and with TOT the products' in tf and tr.  The d_zeta psi
+// sum and the B^(p) solve's matrices both depend on psi only.
+template <class A, class R>
+struct SumMats {
+    A t;
+    Mat2<R> f, r;
+};
+template <bool TOT, class A, class R>
+__device__ __forceinline__ A block_excl_scan_sum_mats1(A t, Mat2<R> mf, Mat2<R> mr, A zero, SumMats<A, R>* sbuf,
+                                                       Mat2<R>& ef, Mat2<R>& er, A& tt, Mat2<R>& tf, Mat2<R>& tr) {
     const Mat2<R> I2 = {1, 0, 0, 1};
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int nw = blockDim.x >> 5;
+    A it = warp_incl_scan<false>(t, OpAdd());
     Mat2<R> ix = warp_incl_scan<false>(mf, OpMatLeft());
     Mat2<R> iy = warp_incl_scan<true>(mr, OpMatLeft());
+    A et = shfl_up_t(it, 1);
     Mat2<R> ex = shfl_up_t(ix, 1), ey = shfl_dn_t(iy, 1);
-    if (lane == 0) ex = I2;
-    if (lane == 31) ey = I2;
-    if (lane == 31) sbuf[warp].x = ix;
-    if (lane == 0) sbuf[warp].y = iy;
+    if (lane == 0) {
+        et = zero;
+        ex = I2;
+        sbuf[warp].r = iy;
+    }
+    if (lane == 31) {
+        ey = I2;
+        sbuf[warp].t = it;
+        sbuf[warp].f = ix;
+    }
     __syncthreads();
-    Mat2<R> wx = lane < nw ? sbuf[lane].x : I2;
-    Mat2<R> wy = lane < nw ? sbuf[lane].y : I2;
-    Mat2<R> sx = warp_incl_scan<false>(wx, OpMatLeft());
-    Mat2<R> sy = warp_incl_scan<true>(wy, OpMatLeft());
+    A wt = zero;
+    Mat2<R> wx = I2, wy = I2;
+    if (lane < nw) {
+        wt = sbuf[lane].t;
+        wx = sbuf[lane].f;
+        wy = sbuf[lane].r;
+    }
+    A st = warp_incl_scan_n<false>(wt, OpAdd(), nw);
+    Mat2<R> sx = warp_incl_scan_n<false>(wx, OpMatLeft(), nw);
+    Mat2<R> sy = warp_incl_scan_n<true>(wy, OpMatLeft(), nw);
+    const int last = scan_last_lane(nw);
+    tt = shfl_idx_t(st, last);
+    A qt = shfl_up_t(st, 1);
     Mat2<R> qx = shfl_up_t(sx, 1), qy = shfl_dn_t(sy, 1);
-    if (lane == 0) qx = I2;
+    if (lane == 0) {
+        qt = zero;
+        qx = I2;
+    }
     if (lane == 31) qy = I2;
     ef = OpMatLeft()(shfl_idx_t(qx, warp), ex);
     er = OpMatLeft()(shfl_idx_t(qy, warp), ey);
     if (TOT) {
-        tf = shfl_idx_t(sx, 31);
+        tf = shfl_idx_t(sx, last);
         tr = shfl_idx_t(sy, 0);
     }
+    return acc_add(shfl_idx_t(qt, warp), et);
 }
 
 // first index i in [0, n) with a[i] >= x (n if none)

@@ -8,14 +8,15 @@
 //     of the previous slice (one exchange at the top of each slice; the AB2
 //     push of a slice waits in the dead region-table arrays and becomes the
 //     state only if no CTA failed the guard);
-//   - the four block-scan totals (each CTA folds the totals of its
-//     predecessors, or successors for the reverse scans, in rank order:
-//     deterministic), the two matrix scans and the two Green's-function sums
-//     sharing one exchange each;
+//   - the block-scan totals (each CTA folds the totals of its predecessors,
+//     or successors for the reverse scans, in rank order: deterministic): the
+//     sums of w and w ln rho, the sum of t with the two matrix products, and
+//     the two Green's-function sums, one exchange each;
 //   - the region table entry just past each CTA's last ring.
-// Beam counting and the fields on beam particles stay inside each CTA: each
-// CTA takes the particles (or query radii) between the previous CTA's last
-// radius and its own, whose rings and regions it holds.  When rings crossed, a local
+// Every ring finds its place among the slice's beam radii, and the fields on
+// beam particles stay inside each CTA: each takes the particles (or query
+// radii) between the previous CTA's last radius and its own, whose rings and
+// regions it holds.  When rings crossed, a local
 // bitonic sort in every CTA is followed by odd-even merge-split rounds
 // between neighbour CTAs (merge path over the two sorted ranges).
 // Every cluster barrier is reached in cluster-uniform control flow.
@@ -112,8 +113,8 @@ __device__ __forceinline__ void fold_rev_shared(const T* recv, int rank, int siz
     __syncthreads();
 }
 
-// shared memory of the cluster march: the fast march's arrays plus one
-// array of per-ring beam counts (which other CTAs add into)
+// shared memory of the cluster march: the fast march's arrays plus one for
+// the merge rounds' copy of the partner's radii
 __host__ __device__ inline size_t cluster_smem_bytes(int T, int K) {
     return fast_smem_bytes(T, K) + 4 * ((size_t)T * K + 8);
 }
@@ -145,8 +146,7 @@ __device__ __forceinline__ bool block_sorted(const float* rh, int nl, int p0) {
 // dead region tables (b, T, D, S, psi; ids in registers) and written back
 // once every CTA has read the old ranges.
 template <int K>
-// scratch: TK words of this CTA's shared memory, zero on entry and on
-// return (the beam count array): the partner's radii are copied there first
+// scratch: TK words of this CTA's shared memory: the partner's radii are copied there first
 // (one DSMEM load per word, in flight together), so that the merge-path
 // search and the merge read them locally instead of one remote load after
 // another.
@@ -193,7 +193,6 @@ __device__ void cluster_merge_round(cg::cluster_group& cl, const FastSmem& sm, i
             }
         }
         __syncthreads();
-        for (int i = tid; i < TK; i += blockDim.x) scratch[i] = 0.f;  // (every search is done)
         const FastSmem A = rmt_sm(cl, sm, left), B = rmt_sm(cl, sm, left + 1);
         for (int l = tid; l < my_n; l += blockDim.x) {
             const int c = code[l];
@@ -248,7 +247,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
     __shared__ float2 s_edges[16];  // every CTA's first and last radius (merge rounds)
     __shared__ int s_stop;
     __shared__ float2 s_nab;       // (a, b) of the next CTA's first region
-    __shared__ Trip<ff> x1[16], f1[2];
+    __shared__ Pair<ff> x1[16], f1[2];
     __shared__ ff x2[16], f2[2];
     __shared__ Mat2<float> x3f[16], x3r[16], f3[4];
     __shared__ ff x4f[16], x4r[16], f4[4];
@@ -285,10 +284,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
     sm.D = sm.T + cap;
     sm.S = sm.D + cap;
     sm.psi = sm.S + cap;
-    // beam particles counted at each ring position; zero between uses (other
-    // CTAs add into it in the distributed count)
-    int32_t* cnt_a = reinterpret_cast<int32_t*>(sm.psi + cap);
-    for (int i = tid; i < cap; i += blockDim.x) cnt_a[i] = 0;
+    float* scratch = sm.psi + cap;  // the merge rounds' copy of the partner's radii
 
     if (tid < CTL_N) s_ctl[tid] = W.ctl[tid];
     cl.sync();  // every CTA has started before any stores into another's shared memory
@@ -473,7 +469,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                 // (csize rounds sort any order; the bound is a safeguard)
                 if (all || round == 2 * csize + 2) break;
                 cl.sync();  // everyone has read the edges before they change
-                cluster_merge_round<K>(cl, sm, n, TK, round & 1, reinterpret_cast<float*>(cnt_a));
+                cluster_merge_round<K>(cl, sm, n, TK, round & 1, scratch);
             }
             if (tid < csize) s_last[tid] = s_edges[tid].y;
         } else if (tid < csize) {
@@ -493,10 +489,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
             ir[k] = __frcp_rn(rh[k]);
         }
 
-        // ---------------- a3: beam particles count into their radial place
-        // (a particle counts at the first ring above it; the particles of
-        // this CTA's rings lie between the previous CTA's last radius and
-        // this CTA's last radius, a contiguous range of the sorted slice)
+        // ---------------- a3: the beam's charge inside each ring
         int b0 = 0, m = 0;
         R qtot = 0;
         if (W.nb > 0 && slice < n_steps) {
@@ -509,24 +502,15 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
         const bool in_stage = stg.cap > 0 && stg.fits(m);
         if (in_stage)
             sb = {stg.arr(sbuf, 0) + (b0 & 3), stg.arr(sbuf, 1) + (b0 & 3), stg.arr(sbuf, 2) + (b0 & 3)};
-        // Two ways, chosen alike by every CTA: when the slice holds at most a
-        // CTA's worth of particles, each CTA counts the particles of its own
-        // rings (those between the previous CTA's last radius and its own);
-        // else the slice's particles are split evenly over the CTAs, which
-        // add into the owning CTA's counts (a cluster barrier then orders the
-        // adds before the scan).  Each thread takes a contiguous run of the
-        // radius-sorted particles, along which ranks and owners only grow,
-        // and adds once per run of particles at the same place.
+        // The radii are searched in shared memory: in the stage, or, for a
+        // slice that was not staged, in a copy in the dead region tables
+        // where they fit them, else where they are.
         __syncthreads();  // (publishes s_last)
-        // Usually the slice's radii fit the dead region tables: they are
-        // staged there and every thread finds, for each of its rings, how
-        // many particles lie strictly below it (a search for the first ring,
-        // short walks for the next); cnt_a then holds that number itself.
-        const bool staged = m > 0 && (in_stage || m <= kFastArrays / 2 * cap);
         const bool dist = m > T && csize > 1;
-        if (staged) {
-            const float* pr = sb.br;
-            if (!in_stage) {  // copied into the dead tables a, b, T, D, S, psi
+        {
+            const bool copied = m > 0 && !in_stage && m <= kFastArrays / 2 * cap;
+            SliceBeam sp = sb;
+            if (copied) {  // into the dead tables a, b, T, D, S, psi
                 float* prw = sm.a;
                 for (int i0 = tid; i0 < m; i0 += kPartBatch * T) {
                     float v[kPartBatch];  // loads in flight together
@@ -537,70 +521,14 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                         if (i0 + j * T < m) prw[i0 + j * T] = v[j];
                 }
                 __syncthreads();
-                pr = prw;
+                sp.br = prw;
             }
-            int L = 0;
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const int p = p0 + k;
-                if (p < nl) {
-                    L = k == 0 ? lower_bound_from(pr, m, 0, rh[k]) : lower_bound_from(pr, m, L, rh[k]);
-                    cnt_a[SW::at(p)] = L;
-                }
-            }
-            __syncthreads();  // the staged radii are overwritten from a5 on
-        } else if (m > 0) {
-            const float* br = sb.br;
-            const int mc = dist ? (m + csize - 1) / csize : m;
-            const int c0q = dist ? crank * mc : 0;
-            const int c1q = dist ? min(m, c0q + mc) : m;
-            const int per = (c1q - c0q + T - 1) / T;
-            const int q0 = c0q + tid * per, q1 = min(c1q, q0 + per);
-            int o = dist ? 0 : crank;                // owner CTA of the current run
-            const float lo_own = crank > 0 ? s_last[crank - 1] : -INFINITY;
-            int lo = 0, at_lo = -1, cnt = 0;
-            bool past = false;
-            for (int qb = q0; qb < q1 && !past; qb += kPartBatch) {
-                float xb[kPartBatch];  // radii loaded together, then walked
-#pragma unroll
-                for (int j = 0; j < kPartBatch; ++j) xb[j] = qb + j < q1 ? br[qb + j] : INFINITY;
-#pragma unroll
-                for (int j = 0; j < kPartBatch; ++j) {
-                    const float x = xb[j];
-                    if (!dist && !(x >= lo_own)) continue;
-                    // owner: the first CTA whose last radius is above x
-                    int o2 = o;
-                    while (o2 < csize && !(x < s_last[o2])) ++o2;
-                    if (o2 >= csize || (!dist && o2 != crank)) {  // beyond (or outside this CTA)
-                        past = true;
-                        break;
-                    }
-                    if (o2 != o) {
-                        if (cnt) atomicAdd(o == crank ? &cnt_a[SW::at(at_lo)] : rmt(cl, &cnt_a[SW::at(at_lo)], o), cnt);
-                        o = o2;
-                        lo = 0;
-                        at_lo = -1;
-                        cnt = 0;
-                    }
-                    const int nl_o = min(TK, n - o * TK);
-                    const float* rh_o = o == crank ? sm.rh : rmt(cl, sm.rh, o);
-                    lo = ring_rank_from<K>(rh_o, nl_o, lo, x, false);
-                    if (lo != at_lo) {
-                        if (cnt) atomicAdd(o == crank ? &cnt_a[SW::at(at_lo)] : rmt(cl, &cnt_a[SW::at(at_lo)], o), cnt);
-                        at_lo = lo;
-                        cnt = 0;
-                    }
-                    ++cnt;
-                }
-            }
-            if (cnt) atomicAdd(o == crank ? &cnt_a[SW::at(at_lo)] : rmt(cl, &cnt_a[SW::at(at_lo)], o), cnt);
-            if (dist) cl.sync();
-            else __syncthreads();
+            ring_beam_field<K>(sp, m, qtot, inv_2pi_dxi, nl - p0, rh, IR, bbv);
+            if (copied) __syncthreads();  // the copy is overwritten from a5 on
         }
 
-        // ---------------- a4: scan of (sum w, sum w ln rho, counts)
+        // ---------------- a4: scan of (sum w, sum w ln rho)
         A sw = zeroA, sl = zeroA;
-        int64_t cnt = 0;
         R lp[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -613,39 +541,34 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                 lp[k] = log1pf(dl * c.ir0);
                 sw = ff_acc(sw, c.w);
                 sl = ff_acc(sl, ff_acc(c.wl0, ff_two_prod(c.w.hi, lp[k])));
-                if (m > 0 && !staged) cnt += cnt_a[a];
             }
         }
-        Trip<A> ex1;
+        Pair<A> ex1;
         A Wtot, Ltot;
         {
-            Trip<A> tot1, pre1, all1;
+            Pair<A> tot1, pre1, all1;
             // (one-barrier scans: a cluster barrier separates each from the next)
-            ex1 = block_excl_scan1<false>(Trip<A>{sw, sl, cnt}, OpAddTrip(), Trip<A>{zeroA, zeroA, 0},
-                                          reinterpret_cast<Trip<A>*>(sscan), tot1);
+            ex1 = block_excl_scan1<false>(Pair<A>{sw, sl}, OpAddPair(), Pair<A>{zeroA, zeroA},
+                                          reinterpret_cast<Pair<A>*>(sscan), tot1);
             cluster_push(cl, x1, tot1);
             cl.sync();
-            fold_fwd_shared(x1, crank, csize, Trip<A>{zeroA, zeroA, 0}, OpAddTrip(), &f1[0], &f1[1]);
+            fold_fwd_shared(x1, crank, csize, Pair<A>{zeroA, zeroA}, OpAddPair(), &f1[0], &f1[1]);
             pre1 = f1[0];
             all1 = f1[1];
-            ex1 = OpAddTrip()(pre1, ex1);
+            ex1 = OpAddPair()(pre1, ex1);
             Wtot = all1.x;
             Ltot = all1.y;
         }
 
-        // ---------------- a5: psi, d_rho psi, psibar, gamma, t; beam field
+        // ---------------- a5: psi, d_rho psi, psibar, gamma, t; the solve's matrices
         A S = ex1.x, L = ex1.y;
         A tl = zeroA;
-        int lb = (int)ex1.c;
+        Mat2<R> Mf = I2, Mb = I2;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             int p = p0 + k;
             if (p < nl) {
                 const int a = SW::at(p);
-                if (m > 0) {
-                    lb = staged ? cnt_a[a] : lb + cnt_a[a];
-                    cnt_a[a] = 0;  // read for the last time this slice
-                }
                 RingConst c = ring_const<K>(ctab, idv[k]);
                 R r = rh[k], u = ur[k];
                 A rf = {r, sm.rl[a]};
@@ -665,9 +588,12 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                 sm.D[a] = ff_to_f(Sm);
                 sm.S[a] = ff_to_f(S);
                 sm.psi[a] = psi;
-                R Q = 0.f;
-                if (m > 0) Q = lb < m ? sb.be[lb] : qtot;
-                bbv[k] = Q * inv_2pi_dxi * IR(k);
+                {
+                    const R wr = c.w.hi * IR(k), hA = 0.5f * (wr * ip);
+                    hav[k] = hA;
+                    Mat2<R> M = {1.f + hA * r, hA * IR(k), -hA * r * r * r, 1.f - hA * r};
+                    Mf = OpMatLeft()(Mf, M);
+                }
                 if (mode == MODE_MARCH && W.dump_psi) {
                     size_t row = (size_t)slice * n + idv[k];
                     W.dump_psi[row] = psi;
@@ -677,23 +603,51 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                 L = ff_acc(L, ff_acc(c.wl0, ff_two_prod(c.w.hi, lp[k])));
                 tl = ff_add_f(tl, tv[k]);
             } else {
-                pbv[k] = 1.f; ipb[k] = 1.f; dprv[k] = 0.f; tv[k] = 0.f; bbv[k] = 0.f;
+                pbv[k] = 1.f; ipb[k] = 1.f; dprv[k] = 0.f; tv[k] = 0.f; hav[k] = 0.f;
+            }
+        }
+#pragma unroll
+        for (int k = K - 1; k >= 0; --k) {
+            if (p0 + k < nl) {
+                R r = rh[k], hA = hav[k];
+                Mat2<R> Mi = {1.f - hA * r, -hA * IR(k), hA * r * r * r, 1.f + hA * r};
+                Mb = OpMatLeft()(Mb, Mi);
             }
         }
         A Tex, Ttot;
+        Mat2<R> Yf, Yb;
         {
-            A Ttot_blk, pre2;
-            Tex = block_excl_scan1<false>(tl, OpAdd(), zeroA, reinterpret_cast<A*>(sscan), Ttot_blk);
-            cluster_push(cl, x2, Ttot_blk);
+            // this CTA's sum and its forward and reverse products go to every CTA
+            A Ttot_blk;
+            Mat2<R> tf, tb;
+            Tex = block_excl_scan_sum_mats1<true>(tl, Mf, Mb, zeroA, reinterpret_cast<SumMats<A, R>*>(sscan), Yf, Yb,
+                                                  Ttot_blk, tf, tb);
+            if (tid < csize) {
+                *rmt(cl, &x2[crank], tid) = Ttot_blk;
+                *rmt(cl, &x3f[crank], tid) = tf;
+                *rmt(cl, &x3r[crank], tid) = tb;
+            }
             cl.sync();
-            fold_fwd_shared(x2, crank, csize, zeroA, OpAdd(), &f2[0], &f2[1]);
-            pre2 = f2[0];
+            // the three folds by one thread each, of different warps where there are as many
+            if (tid == 32 % T) {
+                Mat2<R> pre, all;
+                fold_rev(x3r, crank, csize, I2, OpMatLeft(), pre, all);
+                f3[2] = pre;
+            }
+            if (tid == 64 % T) {
+                A pre, all;
+                fold_fwd(x2, crank, csize, zeroA, OpAdd(), pre, all);
+                f2[0] = pre;
+                f2[1] = all;
+            }
+            fold_fwd_shared(x3f, crank, csize, I2, OpMatLeft(), &f3[0], &f3[1]);
             Ttot = f2[1];
-            Tex = ff_acc(pre2, Tex);
+            Tex = ff_acc(f2[0], Tex);
+            Yf = OpMatLeft()(f3[0], Yf);
+            Yb = OpMatLeft()(f3[2], Yb);
         }
 
         // ---------------- a6 + a7
-        Mat2<R> Mf = I2, Mb = I2;
         {
             A Tacc = Tex;
 #pragma unroll
@@ -716,47 +670,16 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                     R Ac = wr * ip;
                     R Bc = wr * ip2 * (-g * dpr + bbv[k] * pb + uu * dpr * ip - u * dpz) + wr * iR * uu * ip2;
                     R Cc = -wr * (g * ip - 1.f - uu * ip2);
-                    R hA = 0.5f * Ac;
-                    hav[k] = hA;
                     s0v[k] = 0.25f * (2.f * Bc + Ac * Cc);
                     s1v[k] = 0.25f * r * (4.f * Cc - 2.f * Bc * r - Ac * Cc * r);
-                    Mat2<R> M = {1.f + hA * r, hA * iR, -hA * r * r * r, 1.f - hA * r};
-                    Mf = OpMatLeft()(Mf, M);
                     if (mode == MODE_MARCH && W.dump_dpz) W.dump_dpz[(size_t)slice * n + idv[k]] = dpz;
                 } else {
-                    hav[k] = 0.f; s0v[k] = 0.f; s1v[k] = 0.f;
-                }
-            }
-#pragma unroll
-            for (int k = K - 1; k >= 0; --k) {
-                if (p0 + k < nl) {
-                    R r = rh[k], hA = hav[k];
-                    Mat2<R> Mi = {1.f - hA * r, -hA * IR(k), hA * r * r * r, 1.f + hA * r};
-                    Mb = OpMatLeft()(Mb, Mi);
+                    s0v[k] = 0.f; s1v[k] = 0.f;
                 }
             }
         }
 
         // ---------------- a8: B_theta^(p)
-        Mat2<R> Yf, Yb;
-        {
-            // this CTA's forward and reverse products go to every CTA
-            Mat2<R> tf, tb;
-            block_excl_scan_mat_fwd_rev1<true>(Mf, Mb, reinterpret_cast<Pair<Mat2<R>>*>(sscan), Yf, Yb, tf, tb);
-            if (tid < csize) {
-                *rmt(cl, &x3f[crank], tid) = tf;
-                *rmt(cl, &x3r[crank], tid) = tb;
-            }
-            cl.sync();
-            if (tid == 32 % T) {
-                Mat2<R> pre, all;
-                fold_rev(x3r, crank, csize, I2, OpMatLeft(), pre, all);
-                f3[2] = pre;
-            }
-            fold_fwd_shared(x3f, crank, csize, I2, OpMatLeft(), &f3[0], &f3[1]);
-            Yf = OpMatLeft()(f3[0], Yf);
-            Yb = OpMatLeft()(f3[2], Yb);
-        }
         R Rra[K], Rrb[K], Dda[K], Ddb[K];
         {
             Mat2<R> Y = Yf;

@@ -17,17 +17,16 @@
 //
 // Per slice:
 //   a2  sortedness check; bitonic sort of (rho, position) only if needed
-//   a3  beam -> rings: each beam particle of the slice finds its radial
-//       place among the rings (binary search in shared memory) and counts
-//       into it; the count prefix (folded into the first block scan) gives
-//       the enclosed beam charge at every ring
-//   a4  block scan of (sum w, sum w ln rho, counts)
-//   a5  psi, d_rho psi (self weight), psibar, gamma, t
-//   a6  block scan of t -> d_zeta psi
+//   a3  beam -> rings: each ring finds its place among the slice's sorted
+//       beam radii (in shared memory) and the charge prefix there
+//   a4  block scan of (sum w, sum w ln rho)
+//   a5  psi, d_rho psi (self weight), psibar, gamma, t; the 2x2 matrices of
+//       the B_theta^(p) system
+//   a6  block scan of t -> d_zeta psi, with the forward and reverse matrix
+//       products (the regular and the decaying homogeneous solution)
 //   a7  A, B, C and the ring sources of the B_theta^(p) system
-//   a8  B_theta^(p): regular (forward) and decaying (backward) homogeneous
-//       solutions from one forward+reverse 2x2 matrix-product scan, then the
-//       discrete Green's function sums (one forward+reverse scan)
+//   a8  B_theta^(p): the discrete Green's function sums (one forward+reverse
+//       scan)
 //   a9  fields at the slice's beam particles from per-region tables
 //   a10 AB2 push (rho in float-float), axis reflection
 #pragma once
@@ -363,6 +362,27 @@ struct SliceBeam {
     const float* be;   // exclusive charge prefix
 };
 
+// a3: B^(b) at this thread's rings (the first nv of them): how many of the
+// slice's particles lie strictly below a ring, by a search for the first and
+// short walks for the next, and the charge prefix there.
+template <int K, class Inv>
+__device__ __forceinline__ void ring_beam_field(const SliceBeam& sb, int m, float qtot, float inv_2pi_dxi, int nv,
+                                                const float (&rh)[K], const Inv& ir, float (&bbv)[K]) {
+    int L = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        bbv[k] = 0.f;
+        if (k < nv) {
+            float Q = 0.f;
+            if (m > 0) {
+                L = k == 0 ? lower_bound_dev(sb.br, m, rh[0]) : lower_bound_from(sb.br, m, L, rh[k]);
+                Q = L < m ? sb.be[L] : qtot;
+            }
+            bbv[k] = Q * inv_2pi_dxi * ir(k);
+        }
+    }
+}
+
 // Issues the stage of slice s (particles [b0, b0 + m)) if it fits into
 // buffer s & 1; every thread can tell from the offsets whether it was staged.
 __device__ __forceinline__ bool stage_slice(const BeamStage& st, const WakeDev<PrecMixed>& W, int s, int b0, int m,
@@ -426,7 +446,6 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
     sm.D = sm.T + cap;
     sm.S = sm.D + cap;
     sm.psi = sm.S + cap;
-    int32_t* t_cnt = reinterpret_cast<int32_t*>(sm.a);  // beam counts (reuses the a table)
 
     if (tid < CTL_N) s_ctl[tid] = W.ctl[tid];
     __syncthreads();
@@ -543,7 +562,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
             ir[k] = __frcp_rn(rh[k]);
         }
 
-        // ---------------- a3: beam particles count into their radial place
+        // ---------------- a3: the beam's charge inside each ring
         int b0 = 0, m = 0;
         R qtot = 0;
         if (W.nb > 0 && slice < n_steps) {
@@ -565,39 +584,10 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
             const int off = b0 & 3;
             sb = {stg.arr(bf, 0) + off, stg.arr(bf, 1) + off, stg.arr(bf, 2) + off};
         }
-        if (m > 0) {
-            for (int i = tid; i < cap; i += T) t_cnt[i] = 0;
-            __syncthreads();
-            // the first ring strictly above a particle counts it.  Each
-            // thread takes a contiguous run of the slice's radius-sorted
-            // particles (ranks along it only grow) and adds once per run of
-            // particles at the same place.
-            const int per = (m + T - 1) / T;
-            const int q1 = min(m, (tid + 1) * per);
-            int lo = 0, at_lo = -1, cnt = 0;
-            for (int qb = tid * per; qb < q1 && lo < n; qb += kPartBatch) {
-                float xb[kPartBatch];  // radii loaded together, then walked
-#pragma unroll
-                for (int j = 0; j < kPartBatch; ++j) xb[j] = qb + j < q1 ? sb.br[qb + j] : INFINITY;
-#pragma unroll
-                for (int j = 0; j < kPartBatch; ++j) {
-                    lo = ring_rank_from<K>(sm.rh, n, lo, xb[j], false);
-                    if (lo >= n) break;
-                    if (lo != at_lo) {
-                        if (cnt) atomicAdd(&t_cnt[SW::at(at_lo)], cnt);
-                        at_lo = lo;
-                        cnt = 0;
-                    }
-                    ++cnt;
-                }
-            }
-            if (cnt) atomicAdd(&t_cnt[SW::at(at_lo)], cnt);
-            __syncthreads();
-        }
+        ring_beam_field<K>(sb, m, qtot, inv_2pi_dxi, n - p0, rh, IR, bbv);
 
-        // ---------------- a4: scan of (sum w, sum w ln rho, counts)
+        // ---------------- a4: scan of (sum w, sum w ln rho)
         A sw = zeroA, sl = zeroA;
-        int64_t cl = 0;
         R lp[K];  // log1p(delta / rho0)
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -610,26 +600,25 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
                 lp[k] = log1pf(dl * c.ir0);
                 sw = ff_acc(sw, c.w);
                 sl = ff_acc(sl, ff_acc(c.wl0, ff_two_prod(c.w.hi, lp[k])));
-                if (m > 0) cl += t_cnt[a];
             }
         }
-        Trip<A> tot1;
-        // (the four scans of a slice alternate the two halves of sscan: each
+        Pair<A> tot1;
+        // (the three scans of a slice alternate the two halves of sscan: each
         // half is rewritten only after another scan's barrier)
-        Trip<A> ex1 = block_excl_scan1<false>(Trip<A>{sw, sl, cl}, OpAddTrip(), Trip<A>{zeroA, zeroA, 0},
-                                              reinterpret_cast<Trip<A>*>(sscan), tot1);
+        Pair<A> ex1 = block_excl_scan1<false>(Pair<A>{sw, sl}, OpAddPair(), Pair<A>{zeroA, zeroA},
+                                              reinterpret_cast<Pair<A>*>(sscan), tot1);
         const A Wtot = tot1.x, Ltot = tot1.y;
 
-        // ---------------- a5: psi, d_rho psi, psibar, gamma, t; beam field
+        // ---------------- a5: psi, d_rho psi, psibar, gamma, t; the solve's matrices
         A S = ex1.x, L = ex1.y;
         A tl = zeroA;
-        int lb = (int)ex1.c;
+        const Mat2<R> I2 = {1, 0, 0, 1};
+        Mat2<R> Mf = I2, Mb = I2;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             int p = p0 + k;
             if (p < n) {
                 const int a = SW::at(p);
-                if (m > 0) lb += t_cnt[a];  // beam particles strictly below ring p
                 RingConst c = ring_const<K>(ctab, idv[k]);
                 R r = rh[k], u = ur[k];
                 A rf = {r, sm.rl[a]};  // rho in float-float
@@ -651,9 +640,12 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
                 sm.D[a] = ff_to_f(Sm);
                 sm.S[a] = ff_to_f(S);
                 sm.psi[a] = psi;
-                R Q = 0.f;
-                if (m > 0) Q = lb < m ? sb.be[lb] : qtot;
-                bbv[k] = Q * inv_2pi_dxi * IR(k);
+                {
+                    const R wr = c.w.hi * IR(k), hA = 0.5f * (wr * ip);
+                    hav[k] = hA;
+                    Mat2<R> M = {1.f + hA * r, hA * IR(k), -hA * r * r * r, 1.f - hA * r};
+                    Mf = OpMatLeft()(Mf, M);
+                }
                 if (mode == MODE_MARCH && W.dump_psi) {
                     size_t row = (size_t)slice * n + idv[k];
                     W.dump_psi[row] = psi;
@@ -663,15 +655,27 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
                 L = ff_acc(L, ff_acc(c.wl0, ff_two_prod(c.w.hi, lp[k])));
                 tl = ff_add_f(tl, tv[k]);
             } else {
-                pbv[k] = 1.f; ipb[k] = 1.f; dprv[k] = 0.f; tv[k] = 0.f; bbv[k] = 0.f;
+                pbv[k] = 1.f; ipb[k] = 1.f; dprv[k] = 0.f; tv[k] = 0.f; hav[k] = 0.f;
             }
         }
-        A Ttot;
-        A Tex = block_excl_scan1<false>(tl, OpAdd(), zeroA, reinterpret_cast<A*>(sscan + kScanBytes / 2), Ttot);
+#pragma unroll
+        for (int k = K - 1; k >= 0; --k) {
+            if (p0 + k < n) {
+                R r = rh[k], hA = hav[k];
+                Mat2<R> Mi = {1.f - hA * r, -hA * IR(k), hA * r * r * r, 1.f + hA * r};
+                Mb = OpMatLeft()(Mb, Mi);
+            }
+        }
+        A Ttot, Tex;
+        Mat2<R> Yf, Yb;
+        {
+            Mat2<R> tf, tb;
+            Tex = block_excl_scan_sum_mats1<false>(tl, Mf, Mb, zeroA,
+                                                   reinterpret_cast<SumMats<A, R>*>(sscan + kScanBytes / 2), Yf, Yb,
+                                                   Ttot, tf, tb);
+        }
 
         // ---------------- a6 + a7: d_zeta psi, A, B, C, ring sources
-        const Mat2<R> I2 = {1, 0, 0, 1};
-        Mat2<R> Mf = I2, Mb = I2;
         {
             A Tacc = Tex;
 #pragma unroll
@@ -694,33 +698,16 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
                     R Ac = wr * ip;
                     R Bc = wr * ip2 * (-g * dpr + bbv[k] * pb + uu * dpr * ip - u * dpz) + wr * iR * uu * ip2;
                     R Cc = -wr * (g * ip - 1.f - uu * ip2);
-                    R hA = 0.5f * Ac;
-                    hav[k] = hA;
                     s0v[k] = 0.25f * (2.f * Bc + Ac * Cc);
                     s1v[k] = 0.25f * r * (4.f * Cc - 2.f * Bc * r - Ac * Cc * r);
-                    Mat2<R> M = {1.f + hA * r, hA * iR, -hA * r * r * r, 1.f - hA * r};
-                    Mf = OpMatLeft()(Mf, M);
                     if (mode == MODE_MARCH && W.dump_dpz) W.dump_dpz[(size_t)slice * n + idv[k]] = dpz;
                 } else {
-                    hav[k] = 0.f; s0v[k] = 0.f; s1v[k] = 0.f;
-                }
-            }
-#pragma unroll
-            for (int k = K - 1; k >= 0; --k) {
-                if (p0 + k < n) {
-                    R r = rh[k], hA = hav[k];
-                    Mat2<R> Mi = {1.f - hA * r, -hA * IR(k), hA * r * r * r, 1.f + hA * r};
-                    Mb = OpMatLeft()(Mb, Mi);
+                    s0v[k] = 0.f; s1v[k] = 0.f;
                 }
             }
         }
 
         // ---------------- a8: B_theta^(p) region coefficients
-        Mat2<R> Yf, Yb;
-        {
-            Mat2<R> tf, tb;
-            block_excl_scan_mat_fwd_rev1<false>(Mf, Mb, reinterpret_cast<Pair<Mat2<R>>*>(sscan), Yf, Yb, tf, tb);
-        }
         R Rra[K], Rrb[K], Dda[K], Ddb[K];  // R_{p+1}, D_{p+1}
         {
             Mat2<R> Y = Yf;
@@ -766,8 +753,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
         // G_k = sum_{p >= k} gamma_p must be a true suffix sum: a total minus a
         // prefix cancels where G_k is small and multiplies R_k ~ e^rho
         A g_tot, d_tot;
-        Pair<A> gd = block_excl_scan_fwd_rev1(dl, gl, zeroA, reinterpret_cast<Pair<A>*>(sscan + kScanBytes / 2), d_tot,
-                                              g_tot);
+        Pair<A> gd = block_excl_scan_fwd_rev1(dl, gl, zeroA, reinterpret_cast<Pair<A>*>(sscan), d_tot, g_tot);
         {
             R Gk[K];
             A Gsuf = gd.y;  // sum over rings >= p0 + K
