@@ -359,6 +359,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
     uint64_t t_start = 0;
     bool pending_push = false;  // the table arrays a, b, T, D, S hold the push of slice - 1
     bool blk_bad = false;   // this CTA failed the guard at slice - 1
+    int far_skip = 0;       // (resort's memory of rings that moved far)
     int has_prev_before = has_prev;
 
     for (;;) {
@@ -447,8 +448,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
         // ---------------- a2: sort by radius if out of order (cluster-wide)
         if (!all_sorted) {
             // local sort of every CTA's range, then merge-split rounds
-            const int nl_pad = nl < 2 ? 2 : 1 << (32 - __clz(nl - 1));
-            resort<K>(sm, nl, nl_pad, cap);
+            resort<K>(sm, nl, far_skip);
             for (int round = 0;; ++round) {
                 if (tid == 0) {
                     s_edge[0] = sm.rh[SW::at(0)];

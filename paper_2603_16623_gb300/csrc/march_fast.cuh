@@ -144,20 +144,26 @@ __device__ __forceinline__ void ks_bitonic_finish(KeySrc (&v)[K]) {
 // is stable with respect to the previous order, after a push in which rings
 // crossed.  Every thread sorts its K rings' keys in registers, then odd-even
 // merge-split rounds between neighbouring threads' runs move rings up to K
-// places per round, which suffices when rings crossed by few places; after
-// kNearRounds rounds still out of order, a bitonic sort of the same keys.
-// Either way the permutation is the stable sort's.  Keys and indices live in
-// the dead region tables (a..D) and the state is gathered through S and psi,
-// so that it adds few registers to the march loop.
+// places per round, which suffices when rings crossed by few places.  What
+// is still out of order after kNearRounds (inner rings of refined cells move
+// by hundreds of places a slice) is merged pairwise, each thread finding its
+// K outputs by a merge-path search: log2(T) rounds of one barrier, where a
+// bitonic network over the block took log2(n)^2 / 2 (78 for 4096 keys).  A
+// block that had to merge goes straight to it the next kFarSkip times
+// (`skip`).  65,536 rings on 16 blocks: 117 -> 89 us per slice; the blowout
+// wake 17.0 -> 16.9.  Either way the permutation is the stable sort's.  Keys and
+// indices live in the dead region tables (a..D) and the state is gathered
+// through S and psi, so that it adds few registers to the march loop.
 constexpr int kNearRounds = 8;
+constexpr int kFarSkip = 15;
 // beam particles whose radii (and charges) one thread loads together in a3/a9
 constexpr int kPartBatch = 8;
 template <int K>
-__device__ __forceinline__ void resort(const FastSmem& sm, int n, int n_pad, int cap) {
+__device__ __forceinline__ void resort(const FastSmem& sm, int n, int& skip) {
     using SW = Swz<K>;
-    const int T = blockDim.x, tid = threadIdx.x, p0 = tid * K;
-    float* key = sm.a;                                         // [n_pad] over a, b
-    int32_t* idx = reinterpret_cast<int32_t*>(sm.a + 2 * cap);  // [n_pad] over T, D
+    const int T = blockDim.x, tid = threadIdx.x, p0 = tid * K, TK = T * K;
+    float* key = sm.a;  // [TK], swizzled
+    int32_t* idx = reinterpret_cast<int32_t*>(sm.b);
     bool sorted = false;
     {
         KeySrc v[K];
@@ -168,25 +174,31 @@ __device__ __forceinline__ void resort(const FastSmem& sm, int n, int n_pad, int
             v[k].src = p;
         }
         ks_sort<K>(v);
-        for (int round = 0; round <= kNearRounds; ++round) {
+        const int rounds = skip > 0 ? 0 : kNearRounds;
+        for (int round = 0; round <= rounds; ++round) {
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                key[p0 + k] = v[k].key;
-                idx[p0 + k] = v[k].src;
+                const int a = SW::at(p0 + k);
+                key[a] = v[k].key;
+                idx[a] = v[k].src;
             }
             __syncthreads();
-            const bool ok = tid + 1 >= T || !ks_less(KeySrc{key[p0 + K], idx[p0 + K]}, v[K - 1]);
+            bool ok = true;
+            if (tid + 1 < T) {
+                const int a = SW::at(p0 + K);
+                ok = !ks_less(KeySrc{key[a], idx[a]}, v[K - 1]);
+            }
             if (__syncthreads_and(ok)) {
                 sorted = true;
                 break;
             }
-            if (round == kNearRounds) break;
+            if (round == rounds) break;
             const bool left = (tid & 1) == (round & 1);
             const int partner = left ? tid + 1 : tid - 1;
             if (partner >= 0 && partner < T) {
 #pragma unroll
                 for (int k = 0; k < K; ++k) {  // half-cleaner against the partner's run, reversed
-                    const int q = partner * K + (K - 1 - k);
+                    const int q = SW::at(partner * K + (K - 1 - k));
                     const KeySrc w = {key[q], idx[q]};
                     const bool lt = ks_less(v[k], w);
                     if (left ? !lt : lt) v[k] = w;
@@ -196,30 +208,44 @@ __device__ __forceinline__ void resort(const FastSmem& sm, int n, int n_pad, int
             __syncthreads();
         }
     }
-    if (!sorted) {  // bitonic sort of (key, index) from the previous order, padded to n_pad
-        for (int i = tid; i < n_pad; i += T) {
-            key[i] = i < n ? sm.rh[SW::at(i)] : INFINITY;
-            idx[i] = i;
-        }
-        __syncthreads();
-        for (int k2 = 2; k2 <= n_pad; k2 <<= 1) {
-            for (int j = k2 >> 1; j > 0; j >>= 1) {
-                for (int i = tid; i < n_pad; i += T) {
-                    const int ixj = i ^ j;
-                    if (ixj > i) {
-                        const float ki = key[i], kj = key[ixj];
-                        const int vi = idx[i], vj = idx[ixj];
-                        const bool gt = (ki > kj) || (ki == kj && vi > vj);
-                        if (gt == ((i & k2) == 0)) {
-                            key[i] = kj;
-                            key[ixj] = ki;
-                            idx[i] = vj;
-                            idx[ixj] = vi;
-                        }
-                    }
-                }
-                __syncthreads();
+    skip = sorted ? 0 : skip > 0 ? skip - 1 : kFarSkip;
+    if (!sorted) {  // pairwise merges of the threads' runs, from one pair of tables into the other
+        float* key2 = sm.T;
+        int32_t* idx2 = reinterpret_cast<int32_t*>(sm.D);
+        for (int L = K; L < TK; L <<= 1) {
+            const int base = p0 & ~(2 * L - 1), d = p0 - base;
+            const int nA = min(L, TK - base), nB = max(0, min(L, TK - base - L));
+            auto at = [&](int i) {
+                const int a = SW::at(base + i);
+                return KeySrc{key[a], idx[a]};
+            };
+            int lo = max(0, d - nB), hi = min(d, nA);
+            while (lo < hi) {  // outputs before d taken from the first run
+                const int mid = (lo + hi) >> 1;
+                if (ks_less(at(L + d - 1 - mid), at(mid))) hi = mid;
+                else lo = mid + 1;
             }
+            int i = lo, j = d - lo;
+            const KeySrc none = {INFINITY, 0x7fffffff};
+            KeySrc x = i < nA ? at(i) : none, y = j < nB ? at(L + j) : none;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const bool take = !ks_less(y, x);
+                const int a = SW::at(p0 + k);
+                key2[a] = take ? x.key : y.key;
+                idx2[a] = take ? x.src : y.src;
+                if (k + 1 < K) {
+                    if (take) x = ++i < nA ? at(i) : none;
+                    else y = ++j < nB ? at(L + j) : none;
+                }
+            }
+            __syncthreads();
+            float* tk = key;
+            key = key2;
+            key2 = tk;
+            int32_t* ti = idx;
+            idx = idx2;
+            idx2 = ti;
         }
     }
     // gather the state into sorted order, two arrays per pass through S, psi
@@ -230,7 +256,7 @@ __device__ __forceinline__ void resort(const FastSmem& sm, int n, int n_pad, int
         float* x0 = pass == 0 ? sm.rh : pass == 1 ? sm.u : sm.fu;
         float* x1 = pass == 0 ? sm.rl : pass == 1 ? sm.fr : reinterpret_cast<float*>(sm.id);
         for (int i = tid; i < n; i += T) {
-            const int a = SW::at(idx[i]);
+            const int a = SW::at(idx[SW::at(i)]);
             g0[i] = x0[a];
             g1[i] = x1[a];
         }
@@ -517,6 +543,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
 
     const int slice0 = slice;
     uint64_t t_start = 0;
+    int far_skip = 0;
     for (; slice < s_end; ++slice) {
         // time budget (thread 0 decides, read after the order check's barrier)
         if (W.budget_ns > 0 && tid == 0) {
@@ -546,7 +573,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
                 pending |= 1 << ((slice + 1) & 1);
                 stall_armed = false;
             }
-            if (!in_order) resort<K>(sm, n, W.n_pad, cap);
+            if (!in_order) resort<K>(sm, n, far_skip);
         }
 #pragma unroll
         for (int k = 0; k < K; ++k) {
