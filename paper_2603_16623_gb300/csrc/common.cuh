@@ -136,6 +136,9 @@ __device__ __forceinline__ int64_t shfl_up_t(int64_t v, int o) {
 __device__ __forceinline__ int64_t shfl_dn_t(int64_t v, int o) {
     return (int64_t)__shfl_down_sync(0xffffffffu, (long long)v, o);
 }
+__device__ __forceinline__ int32_t shfl_up_t(int32_t v, int o) { return __shfl_up_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ int32_t shfl_dn_t(int32_t v, int o) { return __shfl_down_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ int32_t shfl_idx_t(int32_t v, int l) { return __shfl_sync(0xffffffffu, v, l); }
 __device__ __forceinline__ float shfl_up_t(float v, int o) { return __shfl_up_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ float shfl_dn_t(float v, int o) { return __shfl_down_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ ff shfl_up_t(ff v, int o) { return {shfl_up_t(v.hi, o), shfl_up_t(v.lo, o)}; }

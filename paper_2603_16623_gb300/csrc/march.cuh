@@ -258,7 +258,7 @@ __device__ __forceinline__ ff acc_add_prod(ff a, float x, float y) { return ff_a
 // ---------------------------------------------------------------------------
 constexpr int kMaxWakeCtas = 8;
 constexpr int kMaxPartCtas = 16;                       // (the FP64 on-chip march's largest cluster)
-constexpr int kPartSlot = 64;                          // bytes per block total
+constexpr int kPartSlot = 80;                          // bytes per block total
 constexpr int kPartBuf = kMaxPartCtas * kPartSlot;     // one buffer
 struct WakeCtas {
     int rank = 0, size = 1;

@@ -7,6 +7,7 @@
 #include "march_cluster.cuh"
 #include "march_fast.cuh"
 #include "march_ions.cuh"
+#include "march_reg.cuh"
 #include "march_rk4.cuh"
 
 namespace gbwake {
@@ -34,6 +35,22 @@ F64Shape f64_shape(int32_t n);
 cudaError_t launch_march_f64(const WakeDev<PrecF64>* d_wakes, const int32_t* d_order, int32_t n_wakes,
                              int32_t max_slices, int32_t mode, int32_t threads, int32_t k_rings, int32_t cl,
                              int32_t n_max, cudaStream_t st);
+// the marches with a wake's rings in registers (march_reg.cuh): AB2 with
+// beam grids (or FP64 in blocks of a given size), and RK4; k_rings exactly
+// ceil(n / (threads x cl)), 1 to 4 (above 2 with at most 256 threads; else
+// reg_rings gives 0 and the global-memory marches below serve the wake)
+inline int32_t reg_rings(int32_t n, int32_t threads, int32_t cl) {
+    const int32_t k = (n + threads * cl - 1) / (threads * cl);
+    return k <= 4 && threads <= reg_max_threads(k) ? k : 0;
+}
+template <class P>
+cudaError_t launch_march_reg_ab2(const WakeDev<P>* d_wakes, const int32_t* d_order, int32_t n_wakes,
+                                 int32_t max_slices, int32_t mode, int32_t threads, int32_t k_rings, int32_t cl,
+                                 int32_t n_max, cudaStream_t st);
+template <class P>
+cudaError_t launch_march_reg_rk4(const WakeDev<P>* d_wakes, const int32_t* d_order, int32_t n_wakes,
+                                 int32_t max_slices, int32_t mode, int32_t threads, int32_t k_rings, int32_t cl,
+                                 int32_t n_max, cudaStream_t st);
 // the cluster march: clusters of cl CTAs of `threads` threads, k_rings = 2,
 // 4 or 8 rings per thread
 cudaError_t launch_march_cluster(const WakeDev<PrecMixed>* d_wakes, const int32_t* d_order, int32_t n_wakes,

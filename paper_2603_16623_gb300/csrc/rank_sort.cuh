@@ -23,9 +23,6 @@ namespace gbwake {
 
 __device__ __forceinline__ int32_t radius_key(float r) { return __float_as_int(r); }
 __device__ __forceinline__ int64_t radius_key(double r) { return __double_as_longlong(r); }
-__device__ __forceinline__ int32_t shfl_up_t(int32_t v, int o) { return __shfl_up_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ int32_t shfl_dn_t(int32_t v, int o) { return __shfl_down_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ int32_t shfl_idx_t(int32_t v, int l) { return __shfl_sync(0xffffffffu, v, l); }
 
 struct OpMax {
     template <class T>

@@ -664,6 +664,12 @@ size_t with_ion_own(size_t smem, size_t own) {
 // densest slice, or the most the library accepts when that is not known.
 int32_t stage_want(const wake_handle* h) { return h->slice_max < 0 ? kMaxSliceParticles : h->slice_max; }
 
+// rings per thread of a wake served by the register marches (0: the
+// global-memory marches); wakes of one launch share it
+int32_t gm_reg_rings(const wake_handle* h) {
+    return h->fast_threads || h->n_ion ? 0 : reg_rings(h->n, h->threads, h->gm_cl);
+}
+
 template <class P>
 wake_status launch_one(wake_handle* h, const WakeDev<P>* d_desc, int32_t max_slices, int32_t mode) {
     if constexpr (std::is_same<P, PrecMixed>::value) {
@@ -677,6 +683,11 @@ wake_status launch_one(wake_handle* h, const WakeDev<P>* d_desc, int32_t max_sli
     } else if (h->fast_threads > 0) {
         WK_CUDA(launch_march_f64(d_desc, nullptr, 1, max_slices, mode, h->fast_threads, h->fast_k, h->fast_cl, h->n,
                                  h->st));
+        return WAKE_OK;
+    }
+    if (const int32_t k = gm_reg_rings(h)) {
+        WK_CUDA((h->rk4 ? launch_march_reg_rk4<P> : launch_march_reg_ab2<P>)(
+            d_desc, nullptr, 1, max_slices, mode, h->threads, k, h->gm_cl, h->n, h->st));
         return WAKE_OK;
     }
     int32_t mb_cap = 0;
@@ -875,6 +886,14 @@ wake_status batch_bucket(const std::vector<wake_handle*>& hs, const FastShape& s
         if (e != cudaSuccess) return fail(WAKE_ECUDA, "batched march launch failed: %s", cudaGetErrorString(e));
         return WAKE_OK;
     }
+    if (const int32_t k = gm_reg_rings(hs[0])) {
+        e = (hs[0]->rk4 ? launch_march_reg_rk4<P> : launch_march_reg_ab2<P>)(
+            static_cast<const WakeDev<P>*>(d_buf), d_order, n, max_slices, MODE_MARCH, hs[0]->threads, k,
+            hs[0]->gm_cl, n_max, st);
+        cudaFreeAsync(d_buf, st);
+        if (e != cudaSuccess) return fail(WAKE_ECUDA, "batched march launch failed: %s", cudaGetErrorString(e));
+        return WAKE_OK;
+    }
     int32_t mb_cap = 0;
     size_t smem = march_smem(n_max, pad_max, hs[0]->real_bytes(), kMaxSliceParticles, &mb_cap);
     if (hs[0]->n_ion) {
@@ -972,7 +991,8 @@ std::vector<LaunchGroup> plan_launches(int32_t n, wake_handle* const* hs, bool w
                       (hs[i]->fast_threads ? hs[i]->fast_cl : 0);
         // the one-CTA kernels (plain, two-species, RK4, grids) by their block size
         if (!hs[i]->fast_threads) key = -(1 + (hs[i]->n_ion ? 1 : 0) + 2 * hs[i]->rk4 + 4 * (hs[i]->grid_nr > 0) +
-                                          8 * (hs[i]->threads + 1024 * (hs[i]->gm_cl - 1)));
+                                          8 * (hs[i]->threads + 1024 * (hs[i]->gm_cl - 1 +
+                                                                        kMaxWakeCtas * gm_reg_rings(hs[i]))));
         const double t = predicted_ms(hs[i]);
         int tier = 0;
         while (whole_window && tier + 1 < kTiers && t < kTierFrac[tier] * t_all) ++tier;
