@@ -51,6 +51,15 @@ template <class P>
 cudaError_t launch_march_reg_rk4(const WakeDev<P>* d_wakes, const int32_t* d_order, int32_t n_wakes,
                                  int32_t max_slices, int32_t mode, int32_t threads, int32_t k_rings, int32_t cl,
                                  int32_t n_max, cudaStream_t st);
+// two species (march_reg_ions.cuh): k_rings of each species per thread, 1 or 2
+inline int32_t reg_ion_rings(int32_t n_cells, int32_t threads, int32_t cl) {
+    const int32_t k = (n_cells + threads * cl - 1) / (threads * cl);
+    return k <= 2 ? k : 0;
+}
+template <class P>
+cudaError_t launch_march_reg_ions(const WakeDev<P>* d_wakes, const int32_t* d_order, int32_t n_wakes,
+                                  int32_t max_slices, int32_t mode, int32_t threads, int32_t k_rings, int32_t cl,
+                                  int32_t n_max, cudaStream_t st);
 // the cluster march: clusters of cl CTAs of `threads` threads, k_rings = 2,
 // 4 or 8 rings per thread
 cudaError_t launch_march_cluster(const WakeDev<PrecMixed>* d_wakes, const int32_t* d_order, int32_t n_wakes,

@@ -1,10 +1,10 @@
 // march_reg.cuh -- the AB2 march of beam-grid wakes (and of FP64 wakes of a
 // given block size) and the RK4 march with a wake's rings in registers.
 //
-// The chain and the arithmetic are those of march.cuh and march_rk4.cuh (the
-// same operations in the same order), for shapes of up to 4 rings per thread; the marches there, which keep every per-ring
-// value in global memory, serve shapes of more.  They spent their time on
-// that: ~25 strided reads and writes of per-ring values per ring and
+// The chain and the formulas are those of march.cuh and march_rk4.cuh, for
+// shapes of up to 4 rings per thread; the marches there, which keep every
+// per-ring value in global memory, serve shapes of more.  They spent their
+// time on that: ~25 strided reads and writes of per-ring values per ring and
 // evaluation, each phase waiting for the last one's through L1 or, after a
 // cluster barrier, L2 (long scoreboard first in their profiles), the
 // logarithm, the weights and the quotients hA / r taken two to four times.
@@ -93,6 +93,186 @@ struct Column {
     }
 };
 
+// Eqs. b_coeffs_2, 3: the ring sources B and C of the B_theta^(p) system
+template <class R>
+__device__ __forceinline__ void ring_sources(R w, R r, R u, R pb, R g, R dpr, R dpz, R bb, R& Bc, R& Cc) {
+    const R wr = w / r, pb2 = pb * pb;
+    Bc = -wr * g * dpr / pb2 + wr * bb / pb + (w / (r * r)) * u * u / pb2 + wr * u * u * dpr / (pb2 * pb) -
+         wr * u * dpz / pb2;
+    Cc = -wr * (g / pb - (R)1 - u * u / pb2);
+}
+
+// The jump matrices of a thread's rings multiplied up (Mf, later rings on the
+// left) and their inverses multiplied back (Mb); Ac: Eq. b_coeffs_1, m01 =
+// Ac / (2 r).
+template <int K, class R>
+__device__ __forceinline__ Mat2<R> ring_matrix(R r, R Ac, R m01) {
+    const R hA = (R)0.5 * Ac;
+    return {(R)1 + hA * r, m01, -hA * r * r * r, (R)1 - hA * r};
+}
+template <int K, class R>
+__device__ __forceinline__ Mat2<R> ring_inverse(R r, R Ac, R m01) {
+    const R hA = (R)0.5 * Ac;
+    return {(R)1 - hA * r, -m01, hA * r * r * r, (R)1 + hA * r};
+}
+template <int K, class R>
+__device__ __forceinline__ void ring_products(const R (&r)[K], const R (&Ac)[K], const R (&m01)[K], int np,
+                                              Mat2<R>& Mf, Mat2<R>& Mb) {
+    Mf = Mb = {1, 0, 0, 1};
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if (k < np) Mf = OpMatLeft()(Mf, ring_matrix<K>(r[k], Ac[k], m01[k]));
+#pragma unroll
+    for (int k = K - 1; k >= 0; --k)
+        if (k < np) Mb = OpMatLeft()(Mb, ring_inverse<K>(r[k], Ac[k], m01[k]));
+}
+
+// a8 from the exclusive products Yf, Yb: B^(p) at this thread's rings and
+// b_n; the regions' a, b to the tables where asked.  Takes an exchange and a
+// barrier over the wake, after which the tables are complete.
+template <class P, int K>
+__device__ __forceinline__ void gm_region_solve(const WakeDev<P>& W, WakeCtas& C, GmShared<P>& s, int n, int p0,
+                                                int np, const typename P::R (&r)[K], const typename P::R (&Ac)[K],
+                                                const typename P::R (&m01)[K], const typename P::R (&Bc)[K],
+                                                const typename P::R (&Cc)[K], const Mat2<typename P::R>& Yf,
+                                                const Mat2<typename P::R>& Yb, bool tables, typename P::R (&bp)[K],
+                                                typename P::R& bn) {
+    using R = typename P::R;
+    using A = typename P::A;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const A zeroA = acc_zero(A());
+    // R walked to the end of the rings
+    R Ra[K], Rb[K];
+    {
+        Mat2<R> Y = Yf;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if (k < np) Y = OpMatLeft()(Y, ring_matrix<K>(r[k], Ac[k], m01[k]));
+            Ra[k] = Y.m00;
+            Rb[k] = Y.m10;
+        }
+    }
+    // R at the first region: as the thread before walked it
+    const bool first = C.rank == 0 && tid == 0;
+    R q0 = shfl_up_t(Ra[K - 1], 1), q1 = shfl_up_t(Rb[K - 1], 1);
+    if (lane == 31) {
+        s.edge_r[0][warp] = Ra[K - 1];
+        s.edge_r[1][warp] = Rb[K - 1];
+    }
+    if (C.size > 1 && tid == (int)blockDim.x - 1) {  // for the next block
+        W.Ra[p0 + np] = Ra[K - 1];
+        W.Rb[p0 + np] = Rb[K - 1];
+    }
+    // ---- the Green's sums, D walked back
+    A gl = zeroA, dl = zeroA;
+    R gp[K], dp[K], Da[K], Db[K];
+    {
+        Mat2<R> Y = Yb;
+#pragma unroll
+        for (int k = K - 1; k >= 0; --k)
+            if (k < np) {
+                const R d0 = Y.m01, d1 = Y.m11;
+                const R s0 = (R)0.25 * ((R)2 * Bc[k] + Ac[k] * Cc[k]);
+                const R s1 = (R)0.25 * r[k] * ((R)4 * Cc[k] - (R)2 * Bc[k] * r[k] - Ac[k] * Cc[k] * r[k]);
+                const R wr = Ra[k] * d1 - Rb[k] * d0;
+                gp[k] = (s0 * d1 - s1 * d0) / wr;
+                dp[k] = (Ra[k] * s1 - Rb[k] * s0) / wr;
+                gl = acc_add_r(gl, gp[k]);
+                dl = acc_add_r(dl, dp[k]);
+                Y = OpMatLeft()(Y, ring_inverse<K>(r[k], Ac[k], m01[k]));
+                Da[k] = Y.m01;
+                Db[k] = Y.m11;
+            }
+    }
+    A g_tot, d_tot;
+    Pair<A> gd = block_excl_scan_fwd_rev1(dl, gl, zeroA, s.g, d_tot, g_tot);
+    if (C.size > 1) {
+        const Pair<A>* buf = C.exchange(Pair<A>{d_tot, g_tot});
+        A all;
+        if (tid == 32 % (int)blockDim.x)
+            gm_fold<true>(C, buf, zeroA, OpAdd(), [](Pair<A> v) { return v.y; }, s.pre_g.y, all);
+        if (tid == 0)
+            gm_fold<false>(C, buf, zeroA, OpAdd(), [](Pair<A> v) { return v.x; }, s.pre_g.x, s.tot_g.x);
+        __syncthreads();
+        gd.x = acc_add(s.pre_g.x, gd.x);
+        gd.y = acc_add(s.pre_g.y, gd.y);
+        d_tot = s.tot_g.x;
+    }
+    // ---- a8: the regions' a, b
+    if (lane == 0 && warp > 0) {
+        q0 = s.edge_r[0][warp - 1];
+        q1 = s.edge_r[1][warp - 1];
+    }
+    if (tid == 0 && C.rank > 0 && np > 0) {
+        q0 = W.Ra[p0];
+        q1 = W.Rb[p0];
+    }
+    if (first) {
+        q0 = 1;
+        q1 = 0;
+    }
+    R ak[K], bk[K];
+    {
+        A Gs = gd.y;
+#pragma unroll
+        for (int k = K - 1; k >= 0; --k)
+            if (k < np) {
+                Gs = acc_add_r(Gs, gp[k]);
+                const R G = acc_to_r(Gs);
+                ak[k] = mul_rn(-G, k > 0 ? Ra[k - 1] : q0);
+                bk[k] = mul_rn(-G, k > 0 ? Rb[k - 1] : q1);
+            }
+        A Hex = gd.x;
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (k < np) {
+                const R H = acc_to_r(Hex);
+                ak[k] += H * Da[k];
+                bk[k] += H * Db[k];
+                Hex = acc_add_r(Hex, dp[k]);
+                if (tables) {
+                    W.ak[p0 + k] = ak[k];
+                    W.bk[p0 + k] = bk[k];
+                }
+            }
+    }
+    const R Hn = acc_to_r(d_tot);
+    const R an = mul_rn(Hn, (R)0);  // region n: D_n = (0, 1)
+    bn = mul_rn(Hn, (R)1);
+    if (first && tables) {
+        W.ak[n] = an;
+        W.bk[n] = bn;
+    }
+    if (lane == 0) {
+        s.edge_a[0][warp] = ak[0];
+        s.edge_a[1][warp] = bk[0];
+    }
+    if (C.size > 1 && tid == 0 && np > 0 && !tables) {
+        W.ak[p0] = ak[0];
+        W.bk[p0] = bk[0];
+    }
+    R na = shfl_dn_t(ak[0], 1), nb = shfl_dn_t(bk[0], 1);
+    C.sync();
+    if (lane == 31) {
+        if (tid + 1 < (int)blockDim.x) {
+            na = s.edge_a[0][warp + 1];
+            nb = s.edge_a[1][warp + 1];
+        } else if (p0 + np < n) {
+            na = W.ak[p0 + np];
+            nb = W.bk[p0 + np];
+        }
+    }
+    // B^(p) at the rings
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if (k < np) {
+            const bool end = p0 + k + 1 == n;
+            const R a1 = end ? an : k + 1 < K ? ak[k + 1 < K ? k + 1 : k] : na;
+            const R b1 = end ? bn : k + 1 < K ? bk[k + 1 < K ? k + 1 : k] : nb;
+            bp[k] = (R)0.5 * ((ak[k] + a1) * r[k] + (bk[k] + b1) / r[k]);
+        }
+}
+
 // One evaluation of the fields (a4..a8) at the sorted rings of the wake: this
 // thread's K radii (r, rlo), momenta u, logarithms and weights, and B^(b).
 // `tables`: the region tables are written for the fields at other radii (they
@@ -135,7 +315,6 @@ struct GmFields {
         // ---- a5, and the ring matrices of the B^(p) solve
         A S = ex.x, L = ex.y, tl = zeroA;
         R t[K], Ac[K], m01[K];
-        Mat2<R> Mf = I2, Mb = I2;
 #pragma unroll
         for (int k = 0; k < K; ++k)
             if (k < np) {
@@ -160,18 +339,10 @@ struct GmFields {
                 L = acc_add(L, acc_mul_a(lnr[k], wa[k]));
                 tl = acc_add_r(tl, t[k]);
                 Ac[k] = w / r[k] / pb[k];
-                const R hA = (R)0.5 * Ac[k];
-                m01[k] = hA / r[k];
-                const Mat2<R> M = {(R)1 + hA * r[k], m01[k], -hA * r[k] * r[k] * r[k], (R)1 - hA * r[k]};
-                Mf = OpMatLeft()(Mf, M);
+                m01[k] = (R)0.5 * Ac[k] / r[k];
             }
-#pragma unroll
-        for (int k = K - 1; k >= 0; --k)
-            if (k < np) {
-                const R hA = (R)0.5 * Ac[k];
-                const Mat2<R> Mi = {(R)1 - hA * r[k], -m01[k], hA * r[k] * r[k] * r[k], (R)1 + hA * r[k]};
-                Mb = OpMatLeft()(Mb, Mi);
-            }
+        Mat2<R> Mf, Mb;
+        ring_products<K>(r, Ac, m01, np, Mf, Mb);
         A Ttot;
         Mat2<R> Yf, Yb, tf, tb;
         A Tex = block_excl_scan_sum_mats1<true>(tl, Mf, Mb, zeroA, s.m, Yf, Yb, Ttot, tf, tb);
@@ -192,158 +363,35 @@ struct GmFields {
             Yb = OpMatLeft()(s.pre_r, Yb);
         }
 
-        // ---- a6 + a7, R walked to the end of the rings
-        R Bc[K], Cc[K], Ra[K], Rb[K];
+        // ---- a6 + a7
+        R Bc[K], Cc[K];
         {
             A Tacc = Tex;
-            Mat2<R> Y = Yf;
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
+            for (int k = 0; k < K; ++k)
                 if (k < np) {
                     const R w = acc_hi(wa[k]), wh = acc_hi(wha[k]);
                     if (tables) W.regT[p0 + k] = acc_to_r(acc_sub(Ttot, Tacc));
                     Tacc = acc_add_r(Tacc, t[k]);
                     const R above = acc_to_r(acc_sub(Ttot, Tacc));
                     dpz[k] = -(above + ((R)1 - wh / w) * t[k]);
-                    const R wr = w / r[k], pb2 = pb[k] * pb[k];
-                    Bc[k] = -wr * g[k] * dpr[k] / pb2 + wr * bb[k] / pb[k] + (w / (r[k] * r[k])) * u[k] * u[k] / pb2 +
-                            wr * u[k] * u[k] * dpr[k] / (pb2 * pb[k]) - wr * u[k] * dpz[k] / pb2;
-                    Cc[k] = -wr * (g[k] / pb[k] - (R)1 - u[k] * u[k] / pb2);
-                    const R hA = (R)0.5 * Ac[k];
-                    const Mat2<R> M = {(R)1 + hA * r[k], m01[k], -hA * r[k] * r[k] * r[k], (R)1 - hA * r[k]};
-                    Y = OpMatLeft()(Y, M);
-                }
-                Ra[k] = Y.m00;
-                Rb[k] = Y.m10;
-            }
-        }
-        // R at the first region: as the thread before walked it
-        const bool first = C.rank == 0 && tid == 0;
-        R q0 = shfl_up_t(Ra[K - 1], 1), q1 = shfl_up_t(Rb[K - 1], 1);
-        if (lane == 31) {
-            s.edge_r[0][warp] = Ra[K - 1];
-            s.edge_r[1][warp] = Rb[K - 1];
-        }
-        if (C.size > 1 && tid == (int)blockDim.x - 1) {  // for the next block
-            W.Ra[p0 + np] = Ra[K - 1];
-            W.Rb[p0 + np] = Rb[K - 1];
-        }
-        // ---- the Green's sums, D walked back
-        A gl = zeroA, dl = zeroA;
-        R gp[K], dp[K], Da[K], Db[K];
-        {
-            Mat2<R> Y = Yb;
-#pragma unroll
-            for (int k = K - 1; k >= 0; --k)
-                if (k < np) {
-                    const R hA = (R)0.5 * Ac[k];
-                    const R d0 = Y.m01, d1 = Y.m11;
-                    const R s0 = (R)0.25 * ((R)2 * Bc[k] + Ac[k] * Cc[k]);
-                    const R s1 = (R)0.25 * r[k] * ((R)4 * Cc[k] - (R)2 * Bc[k] * r[k] - Ac[k] * Cc[k] * r[k]);
-                    const R wr = Ra[k] * d1 - Rb[k] * d0;
-                    gp[k] = (s0 * d1 - s1 * d0) / wr;
-                    dp[k] = (Ra[k] * s1 - Rb[k] * s0) / wr;
-                    gl = acc_add_r(gl, gp[k]);
-                    dl = acc_add_r(dl, dp[k]);
-                    const Mat2<R> Mi = {(R)1 - hA * r[k], -m01[k], hA * r[k] * r[k] * r[k], (R)1 + hA * r[k]};
-                    Y = OpMatLeft()(Y, Mi);
-                    Da[k] = Y.m01;
-                    Db[k] = Y.m11;
+                    ring_sources(w, r[k], u[k], pb[k], g[k], dpr[k], dpz[k], bb[k], Bc[k], Cc[k]);
                 }
         }
-        A g_tot, d_tot;
-        Pair<A> gd = block_excl_scan_fwd_rev1(dl, gl, zeroA, s.g, d_tot, g_tot);
-        if (C.size > 1) {
-            const Pair<A>* buf = C.exchange(Pair<A>{d_tot, g_tot});
-            A all;
-            if (tid == 32 % (int)blockDim.x)
-                gm_fold<true>(C, buf, zeroA, OpAdd(), [](Pair<A> v) { return v.y; }, s.pre_g.y, all);
-            if (tid == 0)
-                gm_fold<false>(C, buf, zeroA, OpAdd(), [](Pair<A> v) { return v.x; }, s.pre_g.x, s.tot_g.x);
-            __syncthreads();
-            gd.x = acc_add(s.pre_g.x, gd.x);
-            gd.y = acc_add(s.pre_g.y, gd.y);
-            d_tot = s.tot_g.x;
-        }
-        // ---- a8: the regions' a, b
-        if (lane == 0 && warp > 0) {
-            q0 = s.edge_r[0][warp - 1];
-            q1 = s.edge_r[1][warp - 1];
-        }
-        if (tid == 0 && C.rank > 0 && np > 0) {
-            q0 = W.Ra[p0];
-            q1 = W.Rb[p0];
-        }
-        if (first) {
-            q0 = 1;
-            q1 = 0;
-        }
-        R ak[K], bk[K];
-        {
-            A Gs = gd.y;
-#pragma unroll
-            for (int k = K - 1; k >= 0; --k)
-                if (k < np) {
-                    Gs = acc_add_r(Gs, gp[k]);
-                    const R G = acc_to_r(Gs);
-                    ak[k] = mul_rn(-G, k > 0 ? Ra[k - 1] : q0);
-                    bk[k] = mul_rn(-G, k > 0 ? Rb[k - 1] : q1);
-                }
-            A Hex = gd.x;
-#pragma unroll
-            for (int k = 0; k < K; ++k)
-                if (k < np) {
-                    const R H = acc_to_r(Hex);
-                    ak[k] += H * Da[k];
-                    bk[k] += H * Db[k];
-                    Hex = acc_add_r(Hex, dp[k]);
-                    if (tables) {
-                        W.ak[p0 + k] = ak[k];
-                        W.bk[p0 + k] = bk[k];
-                    }
-                }
-        }
-        const R Hn = acc_to_r(d_tot);
-        const R an = mul_rn(Hn, (R)0), bn = mul_rn(Hn, (R)1);  // region n: D_n = (0, 1)
-        if (first && tables) {
+        if (C.rank == 0 && tid == 0 && tables) {
             W.regS[n] = tot.x;
             W.regL[n] = zeroA;
             W.regT[n] = (R)0;
-            W.ak[n] = an;
-            W.bk[n] = bn;
         }
-        if (lane == 0) {
-            s.edge_a[0][warp] = ak[0];
-            s.edge_a[1][warp] = bk[0];
-        }
-        if (C.size > 1 && tid == 0 && np > 0 && !tables) {
-            W.ak[p0] = ak[0];
-            W.bk[p0] = bk[0];
-        }
-        R na = shfl_dn_t(ak[0], 1), nb = shfl_dn_t(bk[0], 1);
-        C.sync();
-        if (lane == 31) {
-            if (tid + 1 < (int)blockDim.x) {
-                na = s.edge_a[0][warp + 1];
-                nb = s.edge_a[1][warp + 1];
-            } else if (p0 + np < n) {
-                na = W.ak[p0 + np];
-                nb = W.bk[p0 + np];
-            }
-        }
-        // ---- B^(p) at the rings, guard
+        R bn;
+        gm_region_solve<P, K>(W, C, s, n, p0, np, r, Ac, m01, Bc, Cc, Yf, Yb, tables, bp, bn);
+        // ---- guard
         bad = false;
 #pragma unroll
         for (int k = 0; k < K; ++k)
-            if (k < np) {
-                const bool end = p0 + k + 1 == n;
-                const R a1 = end ? an : k + 1 < K ? ak[k + 1 < K ? k + 1 : k] : na;
-                const R b1 = end ? bn : k + 1 < K ? bk[k + 1 < K ? k + 1 : k] : nb;
-                bp[k] = (R)0.5 * ((ak[k] + a1) * r[k] + (bk[k] + b1) / r[k]);
-                if (!(pb[k] > (R)0) || !real_finite(pb[k]) || !real_finite(dpr[k]) || !real_finite(dpz[k]) ||
-                    !real_finite(bp[k]) || !real_finite(bb[k]) || !real_finite(g[k]))
-                    bad = true;
-            }
+            if (k < np && (!(pb[k] > (R)0) || !real_finite(pb[k]) || !real_finite(dpr[k]) || !real_finite(dpz[k]) ||
+                           !real_finite(bp[k]) || !real_finite(bb[k]) || !real_finite(g[k])))
+                bad = true;
     }
 
     // the slice's ring dumps

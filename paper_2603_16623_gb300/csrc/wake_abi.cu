@@ -667,7 +667,14 @@ int32_t stage_want(const wake_handle* h) { return h->slice_max < 0 ? kMaxSlicePa
 // rings per thread of a wake served by the register marches (0: the
 // global-memory marches); wakes of one launch share it
 int32_t gm_reg_rings(const wake_handle* h) {
-    return h->fast_threads || h->n_ion ? 0 : reg_rings(h->n, h->threads, h->gm_cl);
+    if (h->fast_threads) return 0;
+    return h->n_ion ? reg_ion_rings(h->n_ion, h->threads, h->gm_cl) : reg_rings(h->n, h->threads, h->gm_cl);
+}
+template <class P>
+cudaError_t launch_gm_reg(const wake_handle* h, const WakeDev<P>* d_wakes, const int32_t* d_order, int32_t n_wakes,
+                          int32_t max_slices, int32_t mode, int32_t n_max, cudaStream_t st) {
+    auto* launch = h->n_ion ? launch_march_reg_ions<P> : h->rk4 ? launch_march_reg_rk4<P> : launch_march_reg_ab2<P>;
+    return launch(d_wakes, d_order, n_wakes, max_slices, mode, h->threads, gm_reg_rings(h), h->gm_cl, n_max, st);
 }
 
 template <class P>
@@ -685,9 +692,8 @@ wake_status launch_one(wake_handle* h, const WakeDev<P>* d_desc, int32_t max_sli
                                  h->st));
         return WAKE_OK;
     }
-    if (const int32_t k = gm_reg_rings(h)) {
-        WK_CUDA((h->rk4 ? launch_march_reg_rk4<P> : launch_march_reg_ab2<P>)(
-            d_desc, nullptr, 1, max_slices, mode, h->threads, k, h->gm_cl, h->n, h->st));
+    if (gm_reg_rings(h) > 0) {
+        WK_CUDA(launch_gm_reg<P>(h, d_desc, nullptr, 1, max_slices, mode, h->n, h->st));
         return WAKE_OK;
     }
     int32_t mb_cap = 0;
@@ -886,10 +892,8 @@ wake_status batch_bucket(const std::vector<wake_handle*>& hs, const FastShape& s
         if (e != cudaSuccess) return fail(WAKE_ECUDA, "batched march launch failed: %s", cudaGetErrorString(e));
         return WAKE_OK;
     }
-    if (const int32_t k = gm_reg_rings(hs[0])) {
-        e = (hs[0]->rk4 ? launch_march_reg_rk4<P> : launch_march_reg_ab2<P>)(
-            static_cast<const WakeDev<P>*>(d_buf), d_order, n, max_slices, MODE_MARCH, hs[0]->threads, k,
-            hs[0]->gm_cl, n_max, st);
+    if (gm_reg_rings(hs[0]) > 0) {
+        e = launch_gm_reg<P>(hs[0], static_cast<const WakeDev<P>*>(d_buf), d_order, n, max_slices, MODE_MARCH, n_max, st);
         cudaFreeAsync(d_buf, st);
         if (e != cudaSuccess) return fail(WAKE_ECUDA, "batched march launch failed: %s", cudaGetErrorString(e));
         return WAKE_OK;

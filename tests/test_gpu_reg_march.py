@@ -1,7 +1,8 @@
 """The marches with a wake's rings in registers (march_reg.cuh: beam grids,
-RK4, FP64 wakes of a given block size) at every number of rings per thread,
+RK4, FP64 wakes of a given block size; march_reg_ions.cuh: two species) at
+every number of rings per thread,
 full and ragged last blocks, one block and clusters, against the
-global-memory marches that serve more than 4 rings per thread: from a
+global-memory marches that serve more than 4 (2 of each species) rings per thread: from a
 scrambled ring state with equal radii and a ring about to cross the axis,
 two beams, field queries included.
 
@@ -38,12 +39,13 @@ def solve(march, rings, threads, cluster):
     beams = [W.Beam(xi=rng.uniform(-0.01, 0.07, m), r=s * np.abs(rng.standard_normal(m)), w=np.full(m, 0.3 / m))
              for m, s in ((2500, 0.4), (300, 0.02))]
     wk = W.Wake("reg", edges, beams, 0.02, 4, integrator="rk4" if march == "rk4" else "ab2",
+                ions=(1.0, 100.0) if march == "ions" else None,
                 grid_nr=40 if march == "grid" else 600 if march == "wide grid" else 0)
-    centre = 0.5 * (edges[1:] + edges[:-1])
-    rho = np.abs(centre + 0.3 * np.diff(edges) * rng.standard_normal(rings))
+    centre = np.tile(0.5 * (edges[1:] + edges[:-1]), 2 if march == "ions" else 1)
+    rho = np.abs(centre + 0.3 * edges[1] * rng.standard_normal(centre.shape[0]))
     if rings > 2:
         rho[0] = rho[2]
-    ur = 0.05 * rng.standard_normal(rings)
+    ur = 0.05 * rng.standard_normal(centre.shape[0])
     i = int(np.argmin(rho))
     ur[i] = -2.0 * rho[i] / wk.dxi
     kw = {} if march == "ab2" else {"cluster_ctas": cluster}
@@ -75,6 +77,19 @@ def test_register_marches_match_the_global_memory_marches(march, rings):
                 one = 1.0 if f == "psi" else 0.0
                 assert nerr(one + got[part][f], one + ref[part][f]) < TOL, (threads, cluster, part, f)
     assert seen <= {1, 2, 3, 4} or rings == 1024 and 4 in seen
+
+
+@pytest.mark.parametrize("cells", [129, 192, 256, 257, 500, 512])
+def test_register_two_species_march_matches_the_global_memory_march(cells):
+    k, ref = solve("ions", cells, 64, 1)
+    assert k > 4
+    for threads, cluster in ((512, 1), (256, 1), (128, 2), (96, 3), (64, 8)):
+        k, got = solve("ions", cells, threads, cluster)
+        assert k <= 4  # (of both species)
+        for part in got:
+            for f in got[part]:
+                one = 1.0 if f == "psi" else 0.0
+                assert nerr(one + got[part][f], one + ref[part][f]) < TOL, (threads, cluster, part, f)
 
 
 @pytest.mark.parametrize("march", ["ab2", "grid", "rk4"])
