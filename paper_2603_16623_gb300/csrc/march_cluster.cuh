@@ -258,7 +258,8 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
     const int csize = cl.num_blocks();
     const int widx = blockIdx.x / csize;
     const uint64_t t_launch = global_ns();
-    const WakeDev<PrecMixed>& W = wakes[order ? order[widx] : widx];
+    // a query (one wake): every cluster solves the slice and takes its share of the radii
+    const WakeDev<PrecMixed>& W = wakes[mode == MODE_QUERY ? 0 : order ? order[widx] : widx];
     const int T = blockDim.x;
     const int tid = threadIdx.x;
     const int n = W.n;
@@ -894,7 +895,8 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                 // while another still reads them
                 if (dist) cl.sync();
             } else {
-                for (int64_t q = tid; q < W.nq; q += T) {
+                const int64_t q_step = (int64_t)(gridDim.x / csize) * T;
+                for (int64_t q = (int64_t)widx * T + tid; q < W.nq; q += q_step) {
                     const R x = (R)W.rq[q];
                     // a radius belongs here if lo_r < x <= hi_r (CTA 0 also
                     // takes a NaN query, which no comparison places)
@@ -974,6 +976,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
             fail = slice;
         }
     cl.sync();  // no CTA leaves while a peer may still touch its shared memory
+    if (mode == MODE_QUERY) return;  // (the state stays as the march left it: other clusters may still load it)
 
     for (int p = tid; p < nl; p += T) {
         int a = SW::at(p), g = base + p;
@@ -985,8 +988,8 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
         W.rid[buf][g] = sm.id[a];
     }
     if (tid == 0 && crank == 0) {
-        if (mode == MODE_MARCH) put_march_times(W.ctl, t_launch);
-        W.ctl[CTL_NEXT] = mode == MODE_MARCH ? slice : s_ctl[CTL_NEXT];
+        put_march_times(W.ctl, t_launch);
+        W.ctl[CTL_NEXT] = slice;
         W.ctl[CTL_PREV] = has_prev;
         if (status) {
             W.ctl[CTL_STATUS] = status;

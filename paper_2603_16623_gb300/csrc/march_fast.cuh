@@ -449,7 +449,8 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
     __shared__ __align__(8) uint64_t s_bar[2];
 
     const uint64_t t_launch = global_ns();
-    const WakeDev<PrecMixed>& W = wakes[order ? order[blockIdx.x] : blockIdx.x];
+    // a query (one wake): every block solves the slice and takes its share of the radii
+    const WakeDev<PrecMixed>& W = wakes[mode == MODE_QUERY ? 0 : order ? order[blockIdx.x] : blockIdx.x];
     const int T = blockDim.x;
     const int tid = threadIdx.x;
     const int n = W.n;
@@ -888,7 +889,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
             }
         } else {
             const int64_t nq = W.nq;
-            for (int64_t q = tid; q < nq; q += T) {
+            for (int64_t q = (int64_t)blockIdx.x * T + tid; q < nq; q += (int64_t)gridDim.x * T) {
                 R x = (R)W.rq[q];
                 R psi, dpr, dpz, bp, bb = 0.f;
                 if (x > 0.f) {
@@ -957,6 +958,8 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
         __syncthreads();
     }
 
+    if (mode == MODE_QUERY) return;  // (the state stays as the march left it: other blocks may still load it)
+
     // ---- no bulk copy may still write this block's shared memory when it
     // exits: wait (bounded) for any staged slice that was not consumed
     for (int bf = 0; bf < 2; ++bf)
@@ -979,8 +982,8 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
         W.rid[buf][p] = sm.id[a];
     }
     if (tid == 0) {
-        if (mode == MODE_MARCH) put_march_times(W.ctl, t_launch);
-        W.ctl[CTL_NEXT] = mode == MODE_MARCH ? slice : s_ctl[CTL_NEXT];
+        put_march_times(W.ctl, t_launch);
+        W.ctl[CTL_NEXT] = slice;
         W.ctl[CTL_PREV] = has_prev;
         if (status) {
             W.ctl[CTL_STATUS] = status;

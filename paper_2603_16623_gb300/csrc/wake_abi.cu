@@ -677,14 +677,30 @@ cudaError_t launch_gm_reg(const wake_handle* h, const WakeDev<P>* d_wakes, const
     return launch(d_wakes, d_order, n_wakes, max_slices, mode, h->threads, gm_reg_rings(h), h->gm_cl, n_max, st);
 }
 
+// Blocks (clusters of them) that answer an on-chip wake's query of nq radii:
+// each solves the slice itself, in parallel with the others, and takes the
+// radii of its threads, one each until every SM has a block.  A radius is a
+// chain of ~20 dependent loads (its ring, the beam inside it), and in one
+// block a thread's radii followed each other: 20,000 radii of a 2000-ring
+// wake 257 -> 62 us a call (of these the slice ~20, launch and wait ~15; the
+// descriptor from the pool instead of cudaMalloc and cudaFree ~100 of the
+// difference: 100 radii took 180).
+int32_t query_copies(int32_t threads, int32_t cl, int64_t nq) {
+    constexpr int64_t kSms = 152;
+    return (int32_t)std::max<int64_t>(1, std::min((nq + threads - 1) / threads, kSms / cl));
+}
+
+// (mode MODE_QUERY: nq radii in the descriptor)
 template <class P>
-wake_status launch_one(wake_handle* h, const WakeDev<P>* d_desc, int32_t max_slices, int32_t mode) {
+wake_status launch_one(wake_handle* h, const WakeDev<P>* d_desc, int32_t max_slices, int32_t mode, int64_t nq = 0) {
     if constexpr (std::is_same<P, PrecMixed>::value) {
         const int32_t t = h->fast_threads, k = h->fast_k, cl = h->fast_cl;
         if (t > 0) {
             const int32_t stage = march_stage_particles(t, k, cl, stage_want(h));
-            if (cl > 1) WK_CUDA(launch_march_cluster(d_desc, nullptr, 1, max_slices, mode, t, k, cl, stage, h->st));
-            else WK_CUDA(launch_march_fast(d_desc, nullptr, 1, max_slices, mode, t, k, stage, h->st));
+            const int32_t copies = mode == MODE_QUERY ? query_copies(t, cl, nq) : 1;
+            if (cl > 1)
+                WK_CUDA(launch_march_cluster(d_desc, nullptr, copies, max_slices, mode, t, k, cl, stage, h->st));
+            else WK_CUDA(launch_march_fast(d_desc, nullptr, copies, max_slices, mode, t, k, stage, h->st));
             return WAKE_OK;
         }
     } else if (h->fast_threads > 0) {
@@ -737,9 +753,12 @@ wake_status fields_at_impl(wake_handle* h, int64_t n, const double* r, void* ez,
     std::memcpy(&D, h->desc_host.data(), sizeof(D));
     void* outs_user[4] = {ez, wr, bt, psi};
     std::vector<void*> tmp;
-    auto cleanup = [&]() {
-        cudaStreamSynchronize(h->st);
+    void* d_desc = nullptr;  // from the library's pool: a cudaFree would wait for the whole device
+    auto cleanup = [&]() -> cudaError_t {
+        if (d_desc) cudaFreeAsync(d_desc, h->st);
+        const cudaError_t e = cudaStreamSynchronize(h->st);
         for (void* p : tmp) cudaFree(p);
+        return e;
     };
     double* d_r = nullptr;
     if (device_ptrs) {
@@ -772,22 +791,21 @@ wake_status fields_at_impl(wake_handle* h, int64_t n, const double* r, void* ez,
     D.q_wr = d_out[1];
     D.q_bt = d_out[2];
     D.q_psi = d_out[3];
-    void* d_desc = nullptr;
-    if (cudaMalloc(&d_desc, sizeof(D)) != cudaSuccess) {
+    cudaMemPool_t pool = nullptr;
+    if (wake_pool(&pool) != cudaSuccess || cudaMallocFromPoolAsync(&d_desc, sizeof(D), pool, h->st) != cudaSuccess) {
         cudaGetLastError();
+        d_desc = nullptr;
         cleanup();
         return fail(WAKE_ENOMEM, "query descriptor allocation failed");
     }
-    tmp.push_back(d_desc);
     cudaMemcpyAsync(d_desc, &D, sizeof(D), cudaMemcpyHostToDevice, h->st);
-    wake_status s = launch_one<P>(h, static_cast<const WakeDev<P>*>(d_desc), 1, MODE_QUERY);
+    wake_status s = launch_one<P>(h, static_cast<const WakeDev<P>*>(d_desc), 1, MODE_QUERY, n);
     if (s == WAKE_OK && !device_ptrs) {
         for (int k = 0; k < 4; ++k)
             if (outs_user[k])
                 cudaMemcpyAsync(outs_user[k], d_out[k], n * sizeof(R), cudaMemcpyDeviceToHost, h->st);
     }
-    cudaError_t e = cudaStreamSynchronize(h->st);
-    cleanup();
+    const cudaError_t e = cleanup();
     if (s != WAKE_OK) return s;
     if (e != cudaSuccess) return fail(WAKE_ECUDA, "wake_fields_at: %s", cudaGetErrorString(e));
     return WAKE_OK;
@@ -1253,7 +1271,7 @@ wake_status fields_at_static_impl(wake_handle* h, int64_t n, const double* r, vo
         if (d_out[k]) e = cudaMemsetAsync(d_out[k], 0, (size_t)n * sizeof(R), h->st);
     if (e != cudaSuccess)
         return drain(fail(WAKE_ECUDA, "wake_fields_at_static: staging failed: %s", cudaGetErrorString(e)));
-    wake_status s = launch_one<P>(h, reinterpret_cast<const WakeDev<P>*>(base), 1, MODE_QUERY);
+    wake_status s = launch_one<P>(h, reinterpret_cast<const WakeDev<P>*>(base), 1, MODE_QUERY, n);
     if (s != WAKE_OK) return drain(s);
     for (int k = 0; k < 4 && e == cudaSuccess; ++k)
         if (outs_user[k])
