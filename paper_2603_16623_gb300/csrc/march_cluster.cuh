@@ -840,7 +840,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                 const int c1q = dist ? min(m, c0q + mc) : m;
                 const int per = (c1q - c0q + T - 1) / T;
                 const int q0 = c0q + tid * per, q1 = min(c1q, q0 + per);
-                int o = crank, kr = 0;  // owner of the current run and its tables
+                int o = crank, kr = -1;  // owner of the current run and its tables (kr -1: no rank in them yet)
                 FastSmem so = sm;
                 int nl_o = nl;
                 bool past = false;
@@ -870,11 +870,11 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                         o = o2;
                         so = o == crank ? sm : rmt_sm(cl, sm, o);
                         nl_o = min(TK, n - o * TK);
-                        kr = 0;
+                        kr = -1;
                     }
                     R psi, dpr, dpz, bp, bb = 0.f;
                     if (x > 0.f) {
-                        kr = ring_rank_from<K>(so.rh, nl_o, kr, x, true);
+                        kr = kr < 0 ? ring_rank_all<K>(so.rh, nl_o, x) : ring_rank_from<K>(so.rh, nl_o, kr, x, true);
                         fast_fields_region<K>(so, nl_o, TK, kr, x, rmax, half_n, quarter_n, Wtot, Imax, c0, &dpr,
                                               &dpz, &bp, &psi);
                         bb = qb_s[j] * inv_2pi_dxi / x;
