@@ -16,9 +16,8 @@
 // Every ring finds its place among the slice's beam radii, and the fields on
 // beam particles stay inside each CTA: each takes the particles (or query
 // radii) between the previous CTA's last radius and its own, whose rings and
-// regions it holds.  When rings crossed, a local
-// bitonic sort in every CTA is followed by odd-even merge-split rounds
-// between neighbour CTAs (merge path over the two sorted ranges).
+// regions it holds.  When rings crossed, every CTA sorts its own range and
+// the rings that belong to another CTA are counted and moved there.
 // Every cluster barrier is reached in cluster-uniform control flow.
 #pragma once
 
@@ -114,7 +113,7 @@ __device__ __forceinline__ void fold_rev_shared(const T* recv, int rank, int siz
 }
 
 // shared memory of the cluster march: the fast march's arrays plus one for
-// the merge rounds' copy of the partner's radii
+// cluster_move's copies of other CTAs' radii
 __host__ __device__ inline size_t cluster_smem_bytes(int T, int K) {
     return fast_smem_bytes(T, K) + 4 * ((size_t)T * K + 8);
 }
@@ -138,98 +137,128 @@ __device__ __forceinline__ bool block_sorted(const float* rh, int nl, int p0) {
     return __syncthreads_and(ok);
 }
 
-// Odd-even merge-split round between neighbour CTAs (left = even ranks when
-// parity 0, odd when 1): each CTA of a pair rebuilds its range from the merge
-// of the two sorted ranges (ties: left first, which keeps the sort stable).
-// Each thread finds its first merged position by a merge-path search and
-// records where its outputs come from; the state is then gathered into the
-// dead region tables (b, T, D, S, psi; ids in registers) and written back
-// once every CTA has read the old ranges.
+// Moves every ring to its place in the cluster's order, each CTA's own range
+// being sorted already (and without NaN: the places are then a permutation).
+// A ring's place is its position, less the rings of the CTAs before that lie
+// above it, plus the rings of the CTAs after that lie below it (equal radii
+// keep their order, which keeps the sort stable).  Those rings are the last
+// of an earlier CTA's range, the first of a later one's: a warp per CTA finds
+// how many concern this CTA (32 probes at a time, at most 3 too many), their
+// radii are copied to `scratch` (TK words, as many CTAs at a time as fit) and
+// searched there.  The rings are then written to their place in the owner's
+// dead region tables, read back after the one cluster barrier.  Bound by
+// latency (remote loads, barriers): odd-even merge rounds between neighbours,
+// each moving every ring through two cluster barriers, took 24.8k cycles of a
+// 74k-cycle slice with the blocks' own sorts (6000 warm rings on 6 blocks),
+// this 17.2k: the warm restart 5.62 -> 5.21 ms, 65,536 rings 17.7 -> 17.3 ms.
+// s_edges: every CTA's first and last radius; s_last: receives the last
+// radius every CTA then holds.
 template <int K>
-// scratch: TK words of this CTA's shared memory: the partner's radii are copied there first
-// (one DSMEM load per word, in flight together), so that the merge-path
-// search and the merge read them locally instead of one remote load after
-// another.
-__device__ void cluster_merge_round(cg::cluster_group& cl, const FastSmem& sm, int n, int TK, int parity,
-                                    float* scratch) {
+__device__ void cluster_move(cg::cluster_group& cl, const FastSmem& sm, int n, int TK, int nl, float* scratch,
+                             const float2* s_edges, int* s_cnt, float* s_last) {
     using SW = Swz<K>;
     const int rank = cl.block_rank(), size = cl.num_blocks();
-    const int tid = threadIdx.x;
-    int left = -1;
-    if ((rank & 1) == parity && rank + 1 < size) left = rank;
-    else if (rank >= 1 && ((rank - 1) & 1) == parity) left = rank - 1;
-    int32_t* code = reinterpret_cast<int32_t*>(sm.a);  // source: i < nA from A, else nA + j from B
-    int g_id[K];
-    const bool active = left >= 0;
-    int my_n = 0;
-    if (active) {
-        const int nA = min(TK, n - left * TK);
-        const int nB = min(TK, n - (left + 1) * TK);
-        const float* partner = rmt(cl, sm.rh, rank == left ? left + 1 : left);
-        for (int i = tid; i < TK; i += blockDim.x) scratch[i] = partner[i];
-        __syncthreads();  // (active is the same for the whole CTA)
-        const float* Arh = rank == left ? sm.rh : scratch;
-        const float* Brh = rank == left ? scratch : sm.rh;
-        const int off = (rank == left) ? 0 : nA;  // merged position of my local 0
-        my_n = (rank == left) ? nA : nB;
-        const int d = off + tid * K;
-        if (tid * K < my_n) {
-            // merge path: i = number of A elements among the first d merged
-            int lo = max(0, d - nB), hi = min(d, nA);
-            while (lo < hi) {
-                int mid = (lo + hi) >> 1;
-                if (Arh[SW::at(mid)] <= Brh[SW::at(d - 1 - mid)]) lo = mid + 1;
-                else hi = mid;
-            }
-            int i = lo, j = d - lo;
+    const int T = blockDim.x, tid = threadIdx.x, lane = tid & 31, nw = T >> 5;
+    for (int r = tid >> 5; r < size; r += nw) {
+        const bool before = r < rank;
+        const float x = before ? s_edges[rank].x : s_edges[rank].y;
+        int c = 0;
+        if (r != rank && (before ? s_edges[r].y > x : s_edges[r].x < x)) {
+            const int nr = min(TK, n - r * TK);
+            const float* rh = rmt(cl, sm.rh, r);
+            int len = nr - 1;
+            c = 1;  // the count lies in [c, c + len]
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                if (tid * K + k < my_n) {
-                    const bool takeA = i < nA && (j >= nB || Arh[SW::at(i)] <= Brh[SW::at(j)]);
-                    code[tid * K + k] = takeA ? i : nA + j;
-                    if (takeA) ++i;
-                    else ++j;
+            for (int round = 0; round < 2; ++round) {
+                const int step = max(1, (len + 31) / 32), i = c + (lane + 1) * step - 1;
+                bool out = false;  // does ring i, counted from the near end, lie beyond x?
+                if (i < c + len) {
+                    const float v = rh[SW::at(before ? nr - 1 - i : i)];
+                    out = before ? v > x : v < x;
                 }
+                const int some = __popc(__ballot_sync(0xffffffffu, out)) * step;
+                c += some;
+                len = min(step - 1, len - some);
             }
+            c += len;
+        }
+        if (lane == 0) s_cnt[r] = c;
+    }
+    __syncthreads();
+    const int p0 = tid * K, np = max(0, min(K, nl - p0));
+    float x[K];
+    int place[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        x[k] = k < np ? sm.rh[SW::at(p0 + k)] : INFINITY;
+        place[k] = rank * TK + p0 + k;
+    }
+    for (int r0 = 0; r0 < size;) {
+        int r1 = r0, total = 0;
+        while (r1 < size && total + s_cnt[r1] <= TK) total += s_cnt[r1++];  // (a count is at most TK)
+        for (int i = tid; i < total; i += T) {
+            int r = r0, o = i;
+            while (o >= s_cnt[r]) o -= s_cnt[r++];
+            const int at = r < rank ? min(TK, n - r * TK) - s_cnt[r] + o : o;
+            scratch[i] = rmt(cl, sm.rh, r)[SW::at(at)];
         }
         __syncthreads();
-        const FastSmem A = rmt_sm(cl, sm, left), B = rmt_sm(cl, sm, left + 1);
-        for (int l = tid; l < my_n; l += blockDim.x) {
-            const int c = code[l];
-            const FastSmem& S = c < nA ? A : B;
-            const int a = SW::at(c < nA ? c : c - nA);
-            sm.b[l] = S.rh[a];
-            sm.T[l] = S.rl[a];
-            sm.D[l] = S.u[a];
-            sm.S[l] = S.fr[a];
-            sm.psi[l] = S.fu[a];
-        }
+        const float* seg = scratch;
+        for (int r = r0; r < r1; ++r) {
+            const int c = s_cnt[r];
+            const bool before = r < rank;
+            bool any = false;
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int l = tid * K + k;
-            if (l < my_n) {
-                const int c = code[l];
-                g_id[k] = (c < nA ? A : B).id[SW::at(c < nA ? c : c - nA)];
+            for (int k = 0; k < K; ++k)
+                if (k < np && (before ? x[k] < s_edges[r].y : x[k] > s_edges[r].x)) any = true;
+            if (c > 0 && any) {
+                int lo[K];  // how many of the segment lie below x (or at x, before)
+#pragma unroll
+                for (int k = 0; k < K; ++k) lo[k] = 0;
+                for (int len = c; len > 0;) {
+                    const int h = (len + 1) >> 1;
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {
+                        const float v = seg[lo[k] + h - 1];
+                        if (before ? v <= x[k] : v < x[k]) lo[k] += h;
+                    }
+                    len -= h;
+                }
+#pragma unroll
+                for (int k = 0; k < K; ++k) place[k] += before ? lo[k] - c : lo[k];
             }
+            seg += c;
         }
+        r0 = r1;
+        if (r0 < size) __syncthreads();
     }
-    cl.sync();  // every read of the old ranges is done
-    if (active) {
-        for (int l = tid; l < my_n; l += blockDim.x) {
-            const int a = SW::at(l);
-            sm.rh[a] = sm.b[l];
-            sm.rl[a] = sm.T[l];
-            sm.u[a] = sm.D[l];
-            sm.fr[a] = sm.S[l];
-            sm.fu[a] = sm.psi[l];
-        }
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int l = tid * K + k;
-            if (l < my_n) sm.id[SW::at(l)] = g_id[k];
+    for (int k = 0; k < K; ++k) {
+        if (k < np) {
+            const int a = SW::at(p0 + k), r = place[k] / TK, l = place[k] - r * TK, to = SW::at(l);
+            *rmt(cl, &sm.a[to], r) = x[k];
+            *rmt(cl, &sm.b[to], r) = sm.rl[a];
+            *rmt(cl, &sm.T[to], r) = sm.u[a];
+            *rmt(cl, &sm.D[to], r) = sm.fr[a];
+            *rmt(cl, &sm.S[to], r) = sm.fu[a];
+            *rmt(cl, &sm.psi[to], r) = __int_as_float(sm.id[a]);
+            if (l == min(TK, n - r * TK) - 1)
+                for (int q = 0; q < size; ++q) *rmt(cl, &s_last[r], q) = x[k];
         }
     }
-    cl.sync();
+    cl.sync();  // every ring has arrived, every read of the old ranges is done
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        if (k < np) {
+            const int a = SW::at(p0 + k);
+            sm.rh[a] = sm.a[a];
+            sm.rl[a] = sm.b[a];
+            sm.u[a] = sm.T[a];
+            sm.fr[a] = sm.D[a];
+            sm.fu[a] = sm.S[a];
+            sm.id[a] = __float_as_int(sm.psi[a]);
+        }
+    }
 }
 
 template <int K>
@@ -243,8 +272,8 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
     __shared__ int s_ctl[CTL_N];
     __shared__ float4 s_xch[16];   // per rank: (in order?, first radius, last radius, failed the guard?)
     __shared__ float s_last[16];   // last radius held by every CTA, this slice
-    __shared__ float s_edge[2];    // this CTA's first and last radius (merge rounds)
-    __shared__ float2 s_edges[16];  // every CTA's first and last radius (merge rounds)
+    __shared__ float2 s_edges[16];  // every CTA's first and last radius after its own sort
+    __shared__ int s_cnt[16];       // rings of every CTA that cross this CTA's edges
     __shared__ int s_stop;
     __shared__ float2 s_nab;       // (a, b) of the next CTA's first region
     __shared__ Pair<ff> x1[16], f1[2];
@@ -285,7 +314,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
     sm.D = sm.T + cap;
     sm.S = sm.D + cap;
     sm.psi = sm.S + cap;
-    float* scratch = sm.psi + cap;  // the merge rounds' copy of the partner's radii
+    float* scratch = sm.psi + cap;  // cluster_move's copies of other CTAs' radii
 
     if (tid < CTL_N) s_ctl[tid] = W.ctl[tid];
     cl.sync();  // every CTA has started before any stores into another's shared memory
@@ -448,31 +477,29 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
 
         // ---------------- a2: sort by radius if out of order (cluster-wide)
         if (!all_sorted) {
-            // local sort of every CTA's range, then merge-split rounds
+            // local sort of every CTA's range, then every ring to its place
             resort<K>(sm, nl, far_skip);
-            for (int round = 0;; ++round) {
-                if (tid == 0) {
-                    s_edge[0] = sm.rh[SW::at(0)];
-                    s_edge[1] = sm.rh[SW::at(nl - 1)];
-                }
-                cl.sync();
-                // every CTA's edges, one peer per thread (DSMEM loads in
-                // flight together), then the vote from the local copies (the
-                // same for every thread)
-                if (tid < csize) {
-                    const float* e = rmt(cl, s_edge, tid);
-                    s_edges[tid] = make_float2(e[0], e[1]);
-                }
-                __syncthreads();
-                bool all = true;
-                for (int r = 0; r + 1 < csize; ++r)
-                    if (s_edges[r].y > s_edges[r + 1].x) all = false;
-                // (csize rounds sort any order; the bound is a safeguard)
-                if (all || round == 2 * csize + 2) break;
-                cl.sync();  // everyone has read the edges before they change
-                cluster_merge_round<K>(cl, sm, n, TK, round & 1, scratch);
+            // (a NaN radius has no place: its CTA's edges tell, the rings stay,
+            // and the guard stops the wake at this slice)
+            bool nan = false;
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (p0 + k < nl && isnan(sm.rh[SW::at(p0 + k)])) nan = true;
+            nan = __syncthreads_or(nan);
+            // every CTA's edges, pushed to all peers
+            if (tid < csize) {
+                const float none = __int_as_float(0x7fffffff);
+                *rmt(cl, &s_edges[crank], tid) = nan ? make_float2(none, none)
+                                                     : make_float2(sm.rh[SW::at(0)], sm.rh[SW::at(nl - 1)]);
             }
-            if (tid < csize) s_last[tid] = s_edges[tid].y;
+            cl.sync();
+            bool move = false, all_numbers = true;
+            for (int r = 0; r < csize; ++r) {
+                if (isnan(s_edges[r].x)) all_numbers = false;
+                if (r + 1 < csize && s_edges[r].y > s_edges[r + 1].x) move = true;
+            }
+            if (move && all_numbers) cluster_move<K>(cl, sm, n, TK, nl, scratch, s_edges, s_cnt, s_last);
+            else if (tid < csize) s_last[tid] = s_edges[tid].y;
         } else if (tid < csize) {
             s_last[tid] = s_xch[tid].z;
         }
