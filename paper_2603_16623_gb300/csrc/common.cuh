@@ -53,6 +53,7 @@ __device__ __forceinline__ ff ff_acc(ff a, ff b) {
     s.lo = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
     return ff_fast_two_sum(s.hi, s.lo);
 }
+__device__ __forceinline__ ff ff_if(bool on, ff a) { return {on ? a.hi : 0.f, on ? a.lo : 0.f}; }
 __device__ __forceinline__ ff ff_neg(ff a) { return {-a.hi, -a.lo}; }
 __device__ __forceinline__ ff ff_sub(ff a, ff b) { return ff_add(a, ff_neg(b)); }
 __device__ __forceinline__ ff ff_add_f(ff a, float b) {

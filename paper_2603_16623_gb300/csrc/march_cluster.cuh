@@ -296,6 +296,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
     const int base = crank * TK;               // global position of local slot 0
     const int nl = max(0, min(TK, n - base));  // rings held by this CTA (>= 1)
     const int p0 = tid * K;                    // local positions [p0, p0 + K)
+    const int nv = nl - p0;                    // of them the first nv hold rings
     const int cap = TK + 8;
     const bool last_cta = crank == csize - 1;  // holds the last ring and region n
     const RingTab ctab = W.ctab;
@@ -385,6 +386,8 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
         else return ipb[k];
     };
 
+    // (loops over a thread's rings without branches: see march_fast_kernel)
+    const bool dump_fields = mode == MODE_MARCH && W.dump_psi != nullptr;
     const int slice0 = slice;
     uint64_t t_start = 0;
     bool pending_push = false;  // the table arrays a, b, T, D, S hold the push of slice - 1
@@ -505,15 +508,11 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
         }
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            int p = p0 + k;
-            if (p < nl) {
-                int a = SW::at(p);
-                rh[k] = sm.rh[a];
-                ur[k] = sm.u[a];
-                idv[k] = sm.id[a];
-            } else {
-                ur[k] = 0.f; rh[k] = 1.f; idv[k] = 0;
-            }
+            const int a = SW::at(p0 + k);
+            const bool on = k < nv;
+            rh[k] = on ? sm.rh[a] : 1.f;
+            ur[k] = on ? sm.u[a] : 0.f;
+            idv[k] = on ? sm.id[a] : 0;
             ir[k] = __frcp_rn(rh[k]);
         }
 
@@ -551,7 +550,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                 __syncthreads();
                 sp.br = prw;
             }
-            ring_beam_field<K>(sp, m, qtot, inv_2pi_dxi, nl - p0, rh, IR, bbv);
+            ring_beam_field<K>(sp, m, qtot, inv_2pi_dxi, nv, rh, IR, bbv);
             if (copied) __syncthreads();  // the copy is overwritten from a5 on
         }
 
@@ -560,16 +559,14 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
         R lp[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            int p = p0 + k;
-            lp[k] = 0.f;
-            if (p < nl) {
-                const int a = SW::at(p);
-                RingConst c = ring_const<K>(ctab, idv[k]);
-                const R dl = ff_to_f(ff_acc(ff{rh[k], sm.rl[a]}, ff_neg(c.r0)));
-                lp[k] = log1pf(dl * c.ir0);
-                sw = ff_acc(sw, c.w);
-                sl = ff_acc(sl, ff_acc(c.wl0, ff_two_prod(c.w.hi, lp[k])));
-            }
+            const int a = SW::at(p0 + k);
+            const bool on = k < nv;
+            RingConst c = ring_const<K>(ctab, idv[k]);
+            const R dl = ff_to_f(ff_acc(ff{rh[k], sm.rl[a]}, ff_neg(c.r0)));  // rho - rho0
+            const R l1 = log1pf(dl * c.ir0);
+            lp[k] = on ? l1 : 0.f;
+            sw = ff_acc(sw, ff_if(on, c.w));
+            sl = ff_acc(sl, ff_if(on, ff_acc(c.wl0, ff_two_prod(c.w.hi, l1))));
         }
         Pair<A> ex1;
         A Wtot, Ltot;
@@ -622,7 +619,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                     Mat2<R> M = {1.f + hA * r, hA * IR(k), -hA * r * r * r, 1.f - hA * r};
                     Mf = OpMatLeft()(Mf, M);
                 }
-                if (mode == MODE_MARCH && W.dump_psi) {
+                if (K == 2 && mode == MODE_MARCH && W.dump_psi) {
                     size_t row = (size_t)slice * n + idv[k];
                     W.dump_psi[row] = psi;
                     W.dump_dpr[row] = dpr;
@@ -634,13 +631,19 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                 pbv[k] = 1.f; ipb[k] = 1.f; dprv[k] = 0.f; tv[k] = 0.f; hav[k] = 0.f;
             }
         }
+        if (K != 2 && dump_fields)
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (k < nv) {
+                    const size_t row = (size_t)slice * n + idv[k];
+                    W.dump_psi[row] = sm.psi[SW::at(p0 + k)];
+                    W.dump_dpr[row] = dprv[k];
+                }
 #pragma unroll
         for (int k = K - 1; k >= 0; --k) {
-            if (p0 + k < nl) {
-                R r = rh[k], hA = hav[k];
-                Mat2<R> Mi = {1.f - hA * r, -hA * IR(k), hA * r * r * r, 1.f + hA * r};
-                Mb = OpMatLeft()(Mb, Mi);
-            }
+            R r = rh[k], hA = hav[k];
+            Mat2<R> Mi = {1.f - hA * r, -hA * IR(k), hA * r * r * r, 1.f + hA * r};
+            Mb = OpMatLeft()(Mb, Mi);
         }
         A Tex, Ttot;
         Mat2<R> Yf, Yb;
@@ -700,11 +703,15 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                     R Cc = -wr * (g * ip - 1.f - uu * ip2);
                     s0v[k] = 0.25f * (2.f * Bc + Ac * Cc);
                     s1v[k] = 0.25f * r * (4.f * Cc - 2.f * Bc * r - Ac * Cc * r);
-                    if (mode == MODE_MARCH && W.dump_dpz) W.dump_dpz[(size_t)slice * n + idv[k]] = dpz;
+                    if (K == 2 && mode == MODE_MARCH && W.dump_dpz) W.dump_dpz[(size_t)slice * n + idv[k]] = dpz;
                 } else {
                     s0v[k] = 0.f; s1v[k] = 0.f;
                 }
             }
+            if (K != 2 && dump_fields)
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    if (k < nv) W.dump_dpz[(size_t)slice * n + idv[k]] = tv[k];
         }
 
         // ---------------- a8: B_theta^(p)
@@ -713,11 +720,9 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
             Mat2<R> Y = Yf;
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                if (p0 + k < nl) {
-                    R r = rh[k], hA = hav[k];
-                    Mat2<R> M = {1.f + hA * r, hA * IR(k), -hA * r * r * r, 1.f - hA * r};
-                    Y = OpMatLeft()(Y, M);
-                }
+                R r = rh[k], hA = hav[k];
+                Mat2<R> M = {1.f + hA * r, hA * IR(k), -hA * r * r * r, 1.f - hA * r};
+                Y = OpMatLeft()(Y, M);
                 Rra[k] = Y.m00;
                 Rrb[k] = Y.m10;
             }
@@ -815,40 +820,30 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
         R bpv[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            int p = p0 + k;
-            bpv[k] = 0.f;
-            if (p < nl) {
-                const int a = SW::at(p);
-                R a1v, b1v;
-                if (p + 1 < nl) {
-                    int a1 = SW::at(p + 1);
-                    a1v = sm.a[a1];
-                    b1v = sm.b[a1];
-                } else if (last_cta) {  // region n
-                    int a1 = nl < TK ? SW::at(nl) : TK;
-                    a1v = sm.a[a1];
-                    b1v = sm.b[a1];
-                } else {  // first region of the next CTA
-                    a1v = s_nab.x;
-                    b1v = s_nab.y;
-                }
-                R r = rh[k];
-                bpv[k] = 0.5f * ((sm.a[a] + a1v) * r + (sm.b[a] + b1v) * IR(k));
-                R pb = pbv[k];
-                if (!(pb > 0.f) || !isfinite(pb) || !isfinite(dprv[k]) || !isfinite(tv[k]) || !isfinite(bpv[k]) ||
-                    !isfinite(bbv[k]))
-                    bad = true;
-                if (mode == MODE_MARCH) {
-                    size_t row = (size_t)slice * n + idv[k];
-                    if (W.dump_r) W.dump_r[row] = r;
+            const int p = p0 + k, a = SW::at(p);
+            const bool on = k < nv;
+            // the next region: the next ring's, region n, or the next CTA's first
+            const bool in = p + 1 < nl;
+            const int a1 = in ? SW::at(p + 1) : nl < TK ? SW::at(nl) : TK;
+            const R a1v = in || last_cta ? sm.a[a1] : s_nab.x, b1v = in || last_cta ? sm.b[a1] : s_nab.y;
+            const R bp = 0.5f * ((sm.a[a] + a1v) * rh[k] + (sm.b[a] + b1v) * IR(k));
+            bpv[k] = on ? bp : 0.f;
+            const R pb = pbv[k];
+            bad = bad || (on && (!(pb > 0.f) || !isfinite(pb) || !isfinite(dprv[k]) || !isfinite(tv[k]) ||
+                                 !isfinite(bp) || !isfinite(bbv[k])));
+        }
+        if (mode == MODE_MARCH && W.dump_r)
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (k < nv) {
+                    const size_t row = (size_t)slice * n + idv[k];
+                    W.dump_r[row] = rh[k];
                     if (W.dump_ur) {
                         W.dump_ur[row] = ur[k];
                         W.dump_bp[row] = bpv[k];
                         W.dump_bb[row] = bbv[k];
                     }
                 }
-            }
-        }
 
         // ---------------- a9: fields on the beam particles (or query radii)
         // Region k (radii in (rho_{k-1}, rho_k]) lives in the CTA holding
@@ -959,29 +954,21 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
         // failed the guard
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            int p = p0 + k;
-            if (p < nl) {
-                const int a = SW::at(p);
-                R u = ur[k], pb = pbv[k], ip = IPB(k);
-                R g = 0.5f * (1.f + u * u + pb * pb) * ip;
-                R fr = u * ip;
-                R fu = g * dprv[k] * ip - (bpv[k] + bbv[k]);
-                R drr, du;
-                if (has_prev) {
-                    drr = dxi * (1.5f * fr - 0.5f * sm.fr[a]);
-                    du = dxi * (1.5f * fu - 0.5f * sm.fu[a]);
-                } else {
-                    drr = dxi * fr;
-                    du = dxi * fu;
-                }
-                ff rr = ff_add_f(ff{rh[k], sm.rl[a]}, drr);
-                R un = u + du;
-                if (rr.hi < 0.f) {
-                    rr = ff_neg(rr);
-                    un = -un;
-                    fr = -fr;
-                    fu = -fu;
-                }
+            const int a = SW::at(p0 + k);
+            R u = ur[k], pb = pbv[k], ip = IPB(k);
+            R g = 0.5f * (1.f + u * u + pb * pb) * ip;
+            R fr = u * ip;
+            R fu = g * dprv[k] * ip - (bpv[k] + bbv[k]);
+            const R drr = dxi * (has_prev ? 1.5f * fr - 0.5f * sm.fr[a] : fr);
+            const R du = dxi * (has_prev ? 1.5f * fu - 0.5f * sm.fu[a] : fu);
+            ff rr = ff_add_f(ff{rh[k], sm.rl[a]}, drr);
+            R un = u + du;
+            const bool over = rr.hi < 0.f;  // through the axis: the ring reappears at -rho
+            rr = over ? ff_neg(rr) : rr;
+            un = over ? -un : un;
+            fr = over ? -fr : fr;
+            fu = over ? -fu : fu;
+            if (k < nv) {
                 sm.a[a] = rr.hi;
                 sm.b[a] = rr.lo;
                 sm.T[a] = un;

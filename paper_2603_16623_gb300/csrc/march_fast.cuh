@@ -475,6 +475,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
     const int tid = threadIdx.x;
     const int n = W.n;
     const int p0 = tid * K;
+    const int nv = n - p0;  // of the thread's K positions the first nv hold rings
     const int TK = T * K;
     const int cap = TK + 8;
     const RingTab ctab = W.ctab;
@@ -562,6 +563,15 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
         else return ipb[k];
     };
 
+    // The loops over a thread's rings carry no branch per ring where that leaves
+    // every product fused as it was (a position without a ring adds zeros and
+    // identities): a branch keeps the rings' dependent chains from overlapping.
+    // 7700 rings on 8 blocks 22.6 -> 21.2 us per slice, 1800 rings in one 17.6
+    // -> 16.8, both bitwise the same; without a branch in a5, a7 and the
+    // Green's sums too 20.7 and 16.5, but with other products fused, and where
+    // rings cross a last bit grows to 5e-3 of a field.  The dumps stand after
+    // their loops; at 2 rings per thread inside, for the same reason.
+    const bool dump_fields = mode == MODE_MARCH && W.dump_psi != nullptr;
     const int slice0 = slice;
     uint64_t t_start = 0;
     int far_skip = 0;
@@ -598,15 +608,11 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
         }
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            int p = p0 + k;
-            if (p < n) {
-                int a = SW::at(p);
-                rh[k] = sm.rh[a];
-                ur[k] = sm.u[a];
-                idv[k] = sm.id[a];
-            } else {
-                ur[k] = 0.f; rh[k] = 1.f; idv[k] = 0;
-            }
+            const int a = SW::at(p0 + k);
+            const bool on = k < nv;
+            rh[k] = on ? sm.rh[a] : 1.f;
+            ur[k] = on ? sm.u[a] : 0.f;
+            idv[k] = on ? sm.id[a] : 0;
             ir[k] = __frcp_rn(rh[k]);
         }
 
@@ -632,23 +638,21 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
             const int off = b0 & 3;
             sb = {stg.arr(bf, 0) + off, stg.arr(bf, 1) + off, stg.arr(bf, 2) + off};
         }
-        ring_beam_field<K>(sb, m, qtot, inv_2pi_dxi, n - p0, rh, IR, bbv);
+        ring_beam_field<K>(sb, m, qtot, inv_2pi_dxi, nv, rh, IR, bbv);
 
         // ---------------- a4: scan of (sum w, sum w ln rho)
         A sw = zeroA, sl = zeroA;
         R lp[K];  // log1p(delta / rho0)
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            int p = p0 + k;
-            lp[k] = 0.f;
-            if (p < n) {
-                const int a = SW::at(p);
-                RingConst c = ring_const<K>(ctab, idv[k]);
-                const R dl = ff_to_f(ff_acc(ff{rh[k], sm.rl[a]}, ff_neg(c.r0)));  // rho - rho0
-                lp[k] = log1pf(dl * c.ir0);
-                sw = ff_acc(sw, c.w);
-                sl = ff_acc(sl, ff_acc(c.wl0, ff_two_prod(c.w.hi, lp[k])));
-            }
+            const int a = SW::at(p0 + k);
+            const bool on = k < nv;
+            RingConst c = ring_const<K>(ctab, idv[k]);
+            const R dl = ff_to_f(ff_acc(ff{rh[k], sm.rl[a]}, ff_neg(c.r0)));  // rho - rho0
+            const R l1 = log1pf(dl * c.ir0);
+            lp[k] = on ? l1 : 0.f;
+            sw = ff_acc(sw, ff_if(on, c.w));
+            sl = ff_acc(sl, ff_if(on, ff_acc(c.wl0, ff_two_prod(c.w.hi, l1))));
         }
         Pair<A> tot1;
         // (the three scans of a slice alternate the two halves of sscan: each
@@ -694,7 +698,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
                     Mat2<R> M = {1.f + hA * r, hA * IR(k), -hA * r * r * r, 1.f - hA * r};
                     Mf = OpMatLeft()(Mf, M);
                 }
-                if (mode == MODE_MARCH && W.dump_psi) {
+                if (K == 2 && mode == MODE_MARCH && W.dump_psi) {
                     size_t row = (size_t)slice * n + idv[k];
                     W.dump_psi[row] = psi;
                     W.dump_dpr[row] = dpr;
@@ -706,13 +710,19 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
                 pbv[k] = 1.f; ipb[k] = 1.f; dprv[k] = 0.f; tv[k] = 0.f; hav[k] = 0.f;
             }
         }
+        if (K != 2 && dump_fields)
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (k < nv) {
+                    const size_t row = (size_t)slice * n + idv[k];
+                    W.dump_psi[row] = sm.psi[SW::at(p0 + k)];
+                    W.dump_dpr[row] = dprv[k];
+                }
 #pragma unroll
         for (int k = K - 1; k >= 0; --k) {
-            if (p0 + k < n) {
-                R r = rh[k], hA = hav[k];
-                Mat2<R> Mi = {1.f - hA * r, -hA * IR(k), hA * r * r * r, 1.f + hA * r};
-                Mb = OpMatLeft()(Mb, Mi);
-            }
+            R r = rh[k], hA = hav[k];
+            Mat2<R> Mi = {1.f - hA * r, -hA * IR(k), hA * r * r * r, 1.f + hA * r};
+            Mb = OpMatLeft()(Mb, Mi);
         }
         A Ttot, Tex;
         Mat2<R> Yf, Yb;
@@ -748,11 +758,15 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
                     R Cc = -wr * (g * ip - 1.f - uu * ip2);
                     s0v[k] = 0.25f * (2.f * Bc + Ac * Cc);
                     s1v[k] = 0.25f * r * (4.f * Cc - 2.f * Bc * r - Ac * Cc * r);
-                    if (mode == MODE_MARCH && W.dump_dpz) W.dump_dpz[(size_t)slice * n + idv[k]] = dpz;
+                    if (K == 2 && mode == MODE_MARCH && W.dump_dpz) W.dump_dpz[(size_t)slice * n + idv[k]] = dpz;
                 } else {
                     s0v[k] = 0.f; s1v[k] = 0.f;
                 }
             }
+            if (K != 2 && dump_fields)
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    if (k < nv) W.dump_dpz[(size_t)slice * n + idv[k]] = tv[k];
         }
 
         // ---------------- a8: B_theta^(p) region coefficients
@@ -761,11 +775,9 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
             Mat2<R> Y = Yf;
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                if (p0 + k < n) {
-                    R r = rh[k], hA = hav[k];
-                    Mat2<R> M = {1.f + hA * r, hA * IR(k), -hA * r * r * r, 1.f - hA * r};
-                    Y = OpMatLeft()(Y, M);
-                }
+                R r = rh[k], hA = hav[k];
+                Mat2<R> M = {1.f + hA * r, hA * IR(k), -hA * r * r * r, 1.f - hA * r};
+                Y = OpMatLeft()(Y, M);
                 Rra[k] = Y.m00;
                 Rrb[k] = Y.m10;
             }
@@ -847,28 +859,28 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
         R bpv[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            int p = p0 + k;
-            bpv[k] = 0.f;
-            if (p < n) {
-                const int a = SW::at(p);
-                const int a1 = (p + 1 < TK) ? SW::at(p + 1) : TK;
-                R r = rh[k];
-                bpv[k] = 0.5f * ((sm.a[a] + sm.a[a1]) * r + (sm.b[a] + sm.b[a1]) * IR(k));
-                R pb = pbv[k];
-                if (!(pb > 0.f) || !isfinite(pb) || !isfinite(dprv[k]) || !isfinite(tv[k]) || !isfinite(bpv[k]) ||
-                    !isfinite(bbv[k]))
-                    bad = true;
-                if (mode == MODE_MARCH) {
-                    size_t row = (size_t)slice * n + idv[k];
-                    if (W.dump_r) W.dump_r[row] = r;
+            const int p = p0 + k, a = SW::at(p);
+            const bool on = k < nv;
+            const int a1 = p + 1 < TK ? SW::at(p + 1) : TK;
+            const R a1v = sm.a[a1], b1v = sm.b[a1];
+            const R bp = 0.5f * ((sm.a[a] + a1v) * rh[k] + (sm.b[a] + b1v) * IR(k));
+            bpv[k] = on ? bp : 0.f;
+            const R pb = pbv[k];
+            bad = bad || (on && (!(pb > 0.f) || !isfinite(pb) || !isfinite(dprv[k]) || !isfinite(tv[k]) ||
+                                 !isfinite(bp) || !isfinite(bbv[k])));
+        }
+        if (mode == MODE_MARCH && W.dump_r)
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (k < nv) {
+                    const size_t row = (size_t)slice * n + idv[k];
+                    W.dump_r[row] = rh[k];
                     if (W.dump_ur) {
                         W.dump_ur[row] = ur[k];
                         W.dump_bp[row] = bpv[k];
                         W.dump_bb[row] = bbv[k];
                     }
                 }
-            }
-        }
 
         // ---------------- a9: fields on the beam particles (or query radii)
         if (mode == MODE_MARCH) {
@@ -943,29 +955,21 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
         // ---------------- a10: AB2 push (rho in float-float)
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            int p = p0 + k;
-            if (p < n) {
-                const int a = SW::at(p);
-                R u = ur[k], pb = pbv[k], ip = IPB(k);
-                R g = 0.5f * (1.f + u * u + pb * pb) * ip;
-                R fr = u * ip;
-                R fu = g * dprv[k] * ip - (bpv[k] + bbv[k]);
-                R dr, du;
-                if (has_prev) {
-                    dr = dxi * (1.5f * fr - 0.5f * sm.fr[a]);
-                    du = dxi * (1.5f * fu - 0.5f * sm.fu[a]);
-                } else {
-                    dr = dxi * fr;
-                    du = dxi * fu;
-                }
-                ff rr = ff_add_f(ff{rh[k], sm.rl[a]}, dr);
-                R un = u + du;
-                if (rr.hi < 0.f) {  // through the axis: the ring reappears at -rho
-                    rr = ff_neg(rr);
-                    un = -un;
-                    fr = -fr;
-                    fu = -fu;
-                }
+            const int a = SW::at(p0 + k);
+            R u = ur[k], pb = pbv[k], ip = IPB(k);
+            R g = 0.5f * (1.f + u * u + pb * pb) * ip;
+            R fr = u * ip;
+            R fu = g * dprv[k] * ip - (bpv[k] + bbv[k]);
+            const R drr = dxi * (has_prev ? 1.5f * fr - 0.5f * sm.fr[a] : fr);
+            const R du = dxi * (has_prev ? 1.5f * fu - 0.5f * sm.fu[a] : fu);
+            ff rr = ff_add_f(ff{rh[k], sm.rl[a]}, drr);
+            R un = u + du;
+            const bool over = rr.hi < 0.f;  // through the axis: the ring reappears at -rho
+            rr = over ? ff_neg(rr) : rr;
+            un = over ? -un : un;
+            fr = over ? -fr : fr;
+            fu = over ? -fu : fu;
+            if (k < nv) {
                 sm.rh[a] = rr.hi;
                 sm.rl[a] = rr.lo;
                 sm.u[a] = un;
