@@ -29,8 +29,13 @@ cudaError_t launch_slice_sort(const int32_t* off, int32_t n_steps, const double*
                               int32_t* idx, R* br, R* bE, R* bQs, R* bTot, int32_t densest, int32_t* ctl,
                               int32_t* inv, cudaStream_t st);  // inv (nullable): caller index -> sorted position
 template <class R>
-cudaError_t launch_scatter_out(const int32_t* idx, const int32_t* nbin, int64_t nb_max, const R* src, R* dst,
-                               cudaStream_t st);
+struct OutFields {
+    const R* src[4];  // per particle in binned order
+    R* dst[4];        // in the caller's order; null: not wanted
+};
+template <class R>
+cudaError_t launch_scatter_out(const int32_t* idx, const int32_t* nbin, const int32_t* slot, int64_t nb,
+                               const OutFields<R>& f, cudaStream_t st);
 // largest radius of each beam species (caller order, species s = particles
 // [begin[s], begin[s+1])) into rmax[s], which the caller has zeroed
 struct SpeciesRanges {

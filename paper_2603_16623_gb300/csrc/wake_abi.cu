@@ -828,15 +828,19 @@ wake_status beam_fields_enqueue(wake_handle* h, void* const outs_user[4], int32_
             return fail(WAKE_ENOMEM, "beam output staging allocation failed");
         }
     }
+    OutFields<R> f;
+    for (int k = 0; k < 4; ++k) {
+        f.src[k] = static_cast<const R*>(h->d_out[k]);
+        f.dst[k] = device_ptrs ? static_cast<R*>(outs_user[k]) : nullptr;
+    }
     cudaError_t e = cudaSuccess;
-    for (int k = 0; k < 4 && e == cudaSuccess; ++k) {
+    if (device_ptrs) e = launch_scatter_out<R>(h->d_bidx, h->d_boff + h->n_steps, h->d_slot, nb, f, h->st);
+    for (int k = 0; !device_ptrs && k < 4 && e == cudaSuccess; ++k) {  // (one field at a time through the staging)
         if (!outs_user[k]) continue;
-        R* dst = device_ptrs ? static_cast<R*>(outs_user[k]) : tmp;
-        e = cudaMemsetAsync(dst, 0, nb * sizeof(R), h->st);
+        f.dst[k] = tmp;
+        e = launch_scatter_out<R>(h->d_bidx, h->d_boff + h->n_steps, h->d_slot, nb, f, h->st);
+        f.dst[k] = nullptr;
         if (e == cudaSuccess)
-            e = launch_scatter_out<R>(h->d_bidx, h->d_boff + h->n_steps, nb, static_cast<const R*>(h->d_out[k]),
-                                      dst, h->st);
-        if (e == cudaSuccess && !device_ptrs)
             e = cudaMemcpyAsync(outs_user[k], tmp, nb * sizeof(R), cudaMemcpyDeviceToHost, h->st);
     }
     if (tmp) cudaFreeAsync(tmp, h->st);
