@@ -549,9 +549,9 @@ def rk4_bench(args, wakes, stream):
 # warp instructions per ring-slice of the on-chip marches, from the ncu
 # captures summarised in profiles/ (one CTA: 2048 rings, 512 threads x 4;
 # cluster: 6000 rings, 6 CTAs of 256 x 4), and their barriers per slice
-WARP_INSTR_PER_RING_SLICE = {"one_cta": 39.7, "cluster": 48.2}
-BLOCK_BARRIERS_PER_SLICE = {"one_cta": 11, "cluster": 8}
-CLUSTER_BARRIERS_PER_SLICE = 6
+WARP_INSTR_PER_RING_SLICE = {"one_cta": 36.5, "cluster": 43.8}
+BLOCK_BARRIERS_PER_SLICE = {"one_cta": 8, "cluster": 12}
+CLUSTER_BARRIERS_PER_SLICE = 5
 
 
 def latency_roofline(schedule, onchip):

@@ -16,7 +16,7 @@
 // assembled in float-float; everything else is float.
 //
 // Per slice:
-//   a2  sortedness check; bitonic sort of (rho, position) only if needed
+//   a2  sortedness check; re-sort of (rho, position) only if needed
 //   a3  beam -> rings: each ring finds its place among the slice's sorted
 //       beam radii (in shared memory) and the charge prefix there
 //   a4  block scan of (sum w, sum w ln rho)
