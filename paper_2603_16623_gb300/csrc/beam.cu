@@ -79,6 +79,7 @@ __global__ void excl_scan_kernel(const int32_t* __restrict__ cnt, int32_t n, int
 // in the histogram, ranks its particles within each slice in shared memory,
 // reserves one range per non-empty slice with a single global atomic, and
 // writes every index at its slice offset + range start + local rank.
+template <int PER>
 __global__ void bin_scatter_kernel(const int32_t* __restrict__ slot, int64_t n, int32_t n_steps,
                                    const int32_t* __restrict__ off, int32_t* __restrict__ fill,
                                    int32_t* __restrict__ binned_idx) {
@@ -87,9 +88,9 @@ __global__ void bin_scatter_kernel(const int32_t* __restrict__ slot, int64_t n, 
     __syncthreads();
     const int64_t per = (n + gridDim.x - 1) / gridDim.x;
     const int64_t k0 = blockIdx.x * per, k1 = min(n, k0 + per);
-    int32_t rank[kBinPerThread];
+    int32_t rank[PER];
 #pragma unroll
-    for (int j = 0; j < kBinPerThread; ++j) {
+    for (int j = 0; j < PER; ++j) {
         const int64_t k = k0 + threadIdx.x + (int64_t)j * blockDim.x;
         const int32_t s = k < k1 ? slot[k] : -1;
         rank[j] = s >= 0 ? atomicAdd(&hist[s], 1) : -1;
@@ -99,20 +100,24 @@ __global__ void bin_scatter_kernel(const int32_t* __restrict__ slot, int64_t n, 
         if (hist[b]) hist[b] = off[b] + atomicAdd(&fill[b], hist[b]);
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < kBinPerThread; ++j) {
+    for (int j = 0; j < PER; ++j) {
         const int64_t k = k0 + threadIdx.x + (int64_t)j * blockDim.x;
         if (rank[j] >= 0) binned_idx[hist[slot[k]] + rank[j]] = (int32_t)k;
     }
 }
 
 // the slice sort's order: radius, then caller index (distinct but for the
-// padding entries, which go last)
-__device__ __forceinline__ bool kv_less(double ka, int32_t va, double kb, int32_t vb) {
+// padding entries, which go last).  Radii are >= 0, so their bit patterns
+// order as they do and are compared by the integer units: an FP64 comparison
+// holds a sub-partition's FP64 pipe for 64 cycles, and the sort is a chain of
+// them.  With the shorter binning chunks the preparation of a 5500-ring wake
+// with 120k particles 132 -> 106 us, the 48-wake scan 10.60 -> 10.32 ms.
+__device__ __forceinline__ bool kv_less(int64_t ka, int32_t va, int64_t kb, int32_t vb) {
     return ka < kb || (ka == kb && va < vb);
 }
 
 // Sorts keys/vals[0, mp) in shared memory (mp a power of two >= 4, padded
-// with (+inf, INT_MAX)); keys2/vals2 are as large, scratch.  Runs of four
+// with (the largest key, INT_MAX)); keys2/vals2 are as large, scratch.  Runs of four
 // entries are sorted in registers (a bitonic network), then runs of 4, 8,
 // ... are merged pairwise from one buffer into the other: each group of
 // four outputs finds by a merge-path search how many of its predecessors
@@ -122,10 +127,10 @@ __device__ __forceinline__ bool kv_less(double ka, int32_t va, double kb, int32_
 // over the block costs O(mp log^2 mp) with a barrier per stage).  The
 // order is total, so the result is the one sort.
 constexpr int kRun = 4;
-__device__ __forceinline__ void merge_sort_smem(double* keys, int32_t* vals, double* keys2, int32_t* vals2,
+__device__ __forceinline__ void merge_sort_smem(int64_t* keys, int32_t* vals, int64_t* keys2, int32_t* vals2,
                                                 int32_t mp) {
     for (int32_t p0 = (int32_t)threadIdx.x * kRun; p0 < mp; p0 += (int32_t)blockDim.x * kRun) {
-        double k[kRun];
+        int64_t k[kRun];
         int32_t v[kRun];
 #pragma unroll
         for (int e = 0; e < kRun; ++e) {
@@ -140,7 +145,7 @@ __device__ __forceinline__ void merge_sort_smem(double* keys, int32_t* vals, dou
                 for (int i = 0; i < kRun; ++i) {
                     const int l = i ^ j;
                     if (l > i && kv_less(k[l], v[l], k[i], v[i]) == ((i & k2) == 0)) {
-                        const double tk = k[i];
+                        const int64_t tk = k[i];
                         const int32_t tv = v[i];
                         k[i] = k[l];
                         v[i] = v[l];
@@ -155,16 +160,16 @@ __device__ __forceinline__ void merge_sort_smem(double* keys, int32_t* vals, dou
         }
     }
     __syncthreads();
-    double* sk = keys;
+    int64_t* sk = keys;
     int32_t* sv = vals;
-    double* dk = keys2;
+    int64_t* dk = keys2;
     int32_t* dv = vals2;
     for (int32_t L = kRun; L < mp; L <<= 1) {
         for (int32_t p0 = (int32_t)threadIdx.x * kRun; p0 < mp; p0 += (int32_t)blockDim.x * kRun) {
             const int32_t base = p0 & ~(2 * L - 1), d = p0 - base;
-            const double* ak = sk + base;
+            const int64_t* ak = sk + base;
             const int32_t* av = sv + base;
-            const double* bk = ak + L;
+            const int64_t* bk = ak + L;
             const int32_t* bv = av + L;
             int32_t lo = d > L ? d - L : 0, hi = d < L ? d : L;
             while (lo < hi) {  // outputs before d taken from the first run (it goes first on equality)
@@ -188,7 +193,7 @@ __device__ __forceinline__ void merge_sort_smem(double* keys, int32_t* vals, dou
             }
         }
         __syncthreads();
-        double* tk = sk;
+        int64_t* tk = sk;
         sk = dk;
         dk = tk;
         int32_t* tv = sv;
@@ -215,8 +220,9 @@ __global__ void slice_sort_kernel(const int32_t* __restrict__ off, int32_t n_ste
                                   R* __restrict__ bQs, R* __restrict__ bTot, int32_t m_pad, int32_t min_m,
                                   int32_t last, int32_t* __restrict__ ctl, int32_t* __restrict__ inv) {
     extern __shared__ __align__(16) unsigned char smem[];
-    double* keys = reinterpret_cast<double*>(smem);
-    double* pre = keys + m_pad;
+    int64_t* keys = reinterpret_cast<int64_t*>(smem);
+    int64_t* keys2 = keys + m_pad;  // the sort's scratch, then the charge prefix
+    double* pre = reinterpret_cast<double*>(keys2);
     int32_t* vals = reinterpret_cast<int32_t*>(pre + m_pad);
     __shared__ double sbuf[33];
     for (int32_t s = blockIdx.x; s < n_steps; s += gridDim.x) {
@@ -235,15 +241,15 @@ __global__ void slice_sort_kernel(const int32_t* __restrict__ off, int32_t n_ste
         for (int32_t i = threadIdx.x; i < mp; i += blockDim.x) {
             if (i < m) {
                 int32_t k = idx[b0 + i];
-                keys[i] = r_in[k];
+                keys[i] = __double_as_longlong(__dadd_rn(r_in[k], 0.0));  // (-0 to 0)
                 vals[i] = k;
             } else {
-                keys[i] = INFINITY;
+                keys[i] = 0x7fffffffffffffffll;
                 vals[i] = 0x7fffffff;
             }
         }
         __syncthreads();
-        merge_sort_smem(keys, vals, pre, vals + m_pad, mp);
+        merge_sort_smem(keys, vals, keys2, vals + m_pad, mp);
         // exclusive prefix of charge x weight in sorted order (FP64)
         double carry = 0.0;
         for (int32_t base = 0; base < m; base += blockDim.x) {
@@ -260,7 +266,7 @@ __global__ void slice_sort_kernel(const int32_t* __restrict__ off, int32_t n_ste
             while (f > 0 && keys[f - 1] == keys[i]) --f;  // first of a tie group
             idx[b0 + i] = vals[i];
             if (inv) inv[vals[i]] = b0 + i;  // caller index -> sorted position
-            br[b0 + i] = (R)keys[i];
+            br[b0 + i] = (R)__longlong_as_double(keys[i]);
             bE[b0 + i] = (R)pre[i];
             bQs[b0 + i] = (R)pre[f];
         }
@@ -311,9 +317,14 @@ cudaError_t launch_fold_charge(double* qw, const double* w, double q, int64_t n,
     return cudaGetLastError();
 }
 
-// blocks of the binning kernels: chunks of kBinPerThread x 256 particles
+// Blocks of the binning kernels: chunks of 16 x 256 particles, of 4 x 256
+// where those would leave SMs without a block (the slice number's FP64
+// quotient is the count's time, and 120k particles sat on 30 SMs, 17.5 us
+// counted and 13.5 scattered; more blocks than that add only slice counts to
+// merge).
+static bool bin_short(int64_t n) { return n <= (int64_t)152 * 256 * kBinPerThread; }
 static int bin_grid(int64_t n) {
-    const int64_t chunk = (int64_t)kBinPerThread * 256;
+    const int64_t chunk = (int64_t)(bin_short(n) ? kBinPerThreadShort : kBinPerThread) * 256;
     int64_t g = (n + chunk - 1) / chunk;
     return (int)(g < 1 ? 1 : g);
 }
@@ -335,8 +346,8 @@ cudaError_t launch_bin_scatter(const int32_t* slot, int64_t n, int32_t n_steps, 
                                int32_t* binned_idx, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     if (n_steps > kBinSmem) return cudaErrorInvalidValue;
-    bin_scatter_kernel<<<bin_grid(n), 256, (size_t)n_steps * sizeof(int32_t), st>>>(slot, n, n_steps, off, fill,
-                                                                                      binned_idx);
+    auto* kern = bin_short(n) ? bin_scatter_kernel<kBinPerThreadShort> : bin_scatter_kernel<kBinPerThread>;
+    kern<<<bin_grid(n), 256, (size_t)n_steps * sizeof(int32_t), st>>>(slot, n, n_steps, off, fill, binned_idx);
     return cudaGetLastError();
 }
 

@@ -12,7 +12,7 @@ cudaError_t launch_bin_scatter(const int32_t* slot, int64_t n, int32_t n_steps, 
                                int32_t* binned_idx, cudaStream_t st);
 // binning: particles per thread of a block's chunk, and the most slices a
 // window may have (the per-block histogram lives in shared memory)
-constexpr int kBinPerThread = 16;
+constexpr int kBinPerThread = 16, kBinPerThreadShort = 4;
 constexpr int32_t kBinSmem = 48 * 1024 / 4;
 size_t slice_sort_smem(int32_t m_pad);
 // the largest slice the per-slice shared-memory sort takes, and the first
