@@ -20,6 +20,7 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "rank_sort.cuh"
 
 namespace gbwake {
 
@@ -485,8 +486,15 @@ __device__ void bp_region_solve(const WakeDev<P>& W, const typename P::R* sR, in
     }
 }
 
-// Bitonic sort of keys[0..n_pad) ascending, ties by vals ascending (the
-// caller pads with +inf keys); every thread of the block takes part.
+// Bitonic sort of keys[0..n_pad) ascending, ties by vals ascending; every
+// thread of the block takes part.  The caller takes its keys with sort_key
+// and pads with no_ring_key.  Keys are compared by their bit patterns, which
+// order as the radii do and order NaNs too (beyond every number, below the
+// padding): no padding entry comes to lie among the rings, whatever they hold.
+__device__ __forceinline__ float sort_key(float r) { return __fadd_rn(r, 0.f); }  // (-0 to 0)
+__device__ __forceinline__ double sort_key(double r) { return __dadd_rn(r, 0.0); }
+__device__ __forceinline__ float no_ring_key(float) { return __int_as_float(0x7fffffff); }
+__device__ __forceinline__ double no_ring_key(double) { return __longlong_as_double(0x7fffffffffffffffll); }
 template <class R>
 __device__ void block_bitonic_sort(R* keys, int32_t* vals, int n_pad) {
     const int T = blockDim.x, tid = threadIdx.x;
@@ -497,7 +505,8 @@ __device__ void block_bitonic_sort(R* keys, int32_t* vals, int n_pad) {
                 if (ixj > i) {
                     R ki = keys[i], kj = keys[ixj];
                     int vi = vals[i], vj = vals[ixj];
-                    bool gt = (ki > kj) || (ki == kj && vi > vj);
+                    const auto bi = radius_key(ki), bj = radius_key(kj);
+                    bool gt = bi > bj || (bi == bj && vi > vj);
                     if (gt == ((i & k) == 0)) {
                         keys[i] = kj; keys[ixj] = ki;
                         vals[i] = vj; vals[ixj] = vi;
@@ -601,7 +610,7 @@ march_kernel(const WakeDev<P>* __restrict__ wakes, const int32_t* __restrict__ o
             const int nb = buf ^ 1;
             if (sorter) {
                 for (int i = tid; i < W.n_pad; i += T) {
-                    keys[i] = i < n ? rho[i] : (R)INFINITY;
+                    keys[i] = i < n ? sort_key(rho[i]) : no_ring_key(R());
                     vals[i] = i;
                 }
                 __syncthreads();

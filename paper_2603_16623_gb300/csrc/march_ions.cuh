@@ -228,7 +228,7 @@ march_ions_kernel(const WakeDev<P>* __restrict__ wakes, const int32_t* __restric
                     if (C.size > 1 && C.rank != s) continue;
                     const int base = s * N;
                     for (int i = tid; i < W.n_pad; i += T) {
-                        keys[i] = i < N ? rho[base + i] : (R)INFINITY;
+                        keys[i] = i < N ? sort_key(rho[base + i]) : no_ring_key(R());
                         vals[i] = i;
                     }
                     __syncthreads();

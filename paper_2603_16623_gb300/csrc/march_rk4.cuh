@@ -282,7 +282,7 @@ march_rk4_kernel(const WakeDev<P>* __restrict__ wakes, const int32_t* __restrict
                 const int nb = buf ^ 1;
                 if (sorter) {
                     for (int i = tid; i < W.n_pad; i += T) {
-                        keys[i] = i < n ? rho[i] : (R)INFINITY;
+                        keys[i] = i < n ? sort_key(rho[i]) : no_ring_key(R());
                         vals[i] = i;
                     }
                     __syncthreads();
@@ -412,7 +412,7 @@ march_rk4_kernel(const WakeDev<P>* __restrict__ wakes, const int32_t* __restrict
             if (!wake_vote(C, ok, true)) {
                 if (sorter) {
                     for (int i = tid; i < W.n_pad; i += T) {
-                        keys[i] = i < n ? W.rk_r[i] : (R)INFINITY;
+                        keys[i] = i < n ? sort_key(W.rk_r[i]) : no_ring_key(R());
                         vals[i] = i;
                     }
                     __syncthreads();
