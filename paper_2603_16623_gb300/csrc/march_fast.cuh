@@ -31,7 +31,9 @@
 //   a10 AB2 push (rho in float-float), axis reflection
 #pragma once
 
+#include "key_sort.cuh"
 #include "march.cuh"
+#include "rank_sort.cuh"
 #include "stage.cuh"
 
 namespace gbwake {
@@ -97,49 +99,6 @@ struct FastSmem {
     float *a, *b, *T, *D, *S, *psi;  // region tables
 };
 
-// (key, previous position) pairs in the order of the stable sort
-struct KeySrc {
-    float key;
-    int src;
-};
-__device__ __forceinline__ bool ks_less(const KeySrc& a, const KeySrc& b) {
-    return a.key < b.key || (a.key == b.key && a.src < b.src);
-}
-__device__ __forceinline__ void ks_order(KeySrc& a, KeySrc& b) {
-    if (ks_less(b, a)) {
-        KeySrc t = a;
-        a = b;
-        b = t;
-    }
-}
-// sorts v[0, K) ascending (K a power of two): bitonic network, static indices
-template <int K>
-__device__ __forceinline__ void ks_sort(KeySrc (&v)[K]) {
-#pragma unroll
-    for (int k2 = 2; k2 <= K; k2 <<= 1)
-#pragma unroll
-        for (int j = k2 >> 1; j > 0; j >>= 1)
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                const int l = i ^ j;
-                if (l > i) {
-                    if ((i & k2) == 0) ks_order(v[i], v[l]);
-                    else ks_order(v[l], v[i]);
-                }
-            }
-}
-// a bitonic v (after a half-cleaner) into ascending order
-template <int K>
-__device__ __forceinline__ void ks_bitonic_finish(KeySrc (&v)[K]) {
-#pragma unroll
-    for (int j = K >> 1; j > 0; j >>= 1)
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-            const int l = i ^ j;
-            if (l > i) ks_order(v[i], v[l]);
-        }
-}
-
 // Re-sort of the ring state by (rho, previous position), i.e. the sort that
 // is stable with respect to the previous order, after a push in which rings
 // crossed.  Every thread sorts its K rings' keys in registers, then odd-even
@@ -162,7 +121,7 @@ template <int K>
 __device__ __forceinline__ void resort(const FastSmem& sm, int n, int& skip) {
     using SW = Swz<K>;
     const int T = blockDim.x, tid = threadIdx.x, p0 = tid * K, TK = T * K;
-    float* key = sm.a;  // [TK], swizzled
+    int32_t* key = reinterpret_cast<int32_t*>(sm.a);  // [TK], swizzled
     int32_t* idx = reinterpret_cast<int32_t*>(sm.b);
     bool sorted = false;
     {
@@ -170,7 +129,7 @@ __device__ __forceinline__ void resort(const FastSmem& sm, int n, int& skip) {
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int p = p0 + k;
-            v[k].key = p < n ? sm.rh[SW::at(p)] : INFINITY;
+            v[k].key = p < n ? radius_key(__fadd_rn(sm.rh[SW::at(p)], 0.f)) : kNoRingKey;  // (-0 to 0)
             v[k].src = p;
         }
         ks_sort<K>(v);
@@ -196,51 +155,33 @@ __device__ __forceinline__ void resort(const FastSmem& sm, int n, int& skip) {
             const bool left = (tid & 1) == (round & 1);
             const int partner = left ? tid + 1 : tid - 1;
             if (partner >= 0 && partner < T) {
-#pragma unroll
-                for (int k = 0; k < K; ++k) {  // half-cleaner against the partner's run, reversed
-                    const int q = SW::at(partner * K + (K - 1 - k));
-                    const KeySrc w = {key[q], idx[q]};
-                    const bool lt = ks_less(v[k], w);
-                    if (left ? !lt : lt) v[k] = w;
-                }
-                ks_bitonic_finish<K>(v);
+                ks_merge_split<K>(v, [&](int k) {
+                    const int q = SW::at(partner * K + k);
+                    return KeySrc{key[q], idx[q]};
+                }, left);
             }
             __syncthreads();
         }
     }
     skip = sorted ? 0 : skip > 0 ? skip - 1 : kFarSkip;
     if (!sorted) {  // pairwise merges of the threads' runs, from one pair of tables into the other
-        float* key2 = sm.T;
+        int32_t* key2 = reinterpret_cast<int32_t*>(sm.T);
         int32_t* idx2 = reinterpret_cast<int32_t*>(sm.D);
         for (int L = K; L < TK; L <<= 1) {
-            const int base = p0 & ~(2 * L - 1), d = p0 - base;
-            const int nA = min(L, TK - base), nB = max(0, min(L, TK - base - L));
-            auto at = [&](int i) {
-                const int a = SW::at(base + i);
-                return KeySrc{key[a], idx[a]};
-            };
-            int lo = max(0, d - nB), hi = min(d, nA);
-            while (lo < hi) {  // outputs before d taken from the first run
-                const int mid = (lo + hi) >> 1;
-                if (ks_less(at(L + d - 1 - mid), at(mid))) hi = mid;
-                else lo = mid + 1;
-            }
-            int i = lo, j = d - lo;
-            const KeySrc none = {INFINITY, 0x7fffffff};
-            KeySrc x = i < nA ? at(i) : none, y = j < nB ? at(L + j) : none;
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const bool take = !ks_less(y, x);
-                const int a = SW::at(p0 + k);
-                key2[a] = take ? x.key : y.key;
-                idx2[a] = take ? x.src : y.src;
-                if (k + 1 < K) {
-                    if (take) x = ++i < nA ? at(i) : none;
-                    else y = ++j < nB ? at(L + j) : none;
-                }
-            }
+            const int base = p0 & ~(2 * L - 1);
+            ks_merge_outputs<K>(
+                [&](int i) {
+                    const int a = SW::at(base + i);
+                    return KeySrc{key[a], idx[a]};
+                },
+                L, min(L, TK - base), max(0, min(L, TK - base - L)), p0 - base,
+                [&](int k, KeySrc e) {
+                    const int a = SW::at(p0 + k);
+                    key2[a] = e.key;
+                    idx2[a] = e.src;
+                });
             __syncthreads();
-            float* tk = key;
+            int32_t* tk = key;
             key = key2;
             key2 = tk;
             int32_t* ti = idx;

@@ -19,8 +19,12 @@ def _gpu():
     yield
 
 
-# the global-memory and the register marches of every kind, FP64 on chip (one block, a cluster)
+# one block at 2, 4, 8 rings per thread; clusters at 4, 2, 8; FP64 on chip (one block, a cluster); the register and the
+# global-memory marches of every kind
 CASES = [
+    ("ab2", "mixed", 200, {}), ("ab2", "mixed", 1500, {}), ("ab2", "mixed", 2000, dict(rings_per_thread=8, cluster_ctas=1)),
+    ("ab2", "mixed", 3000, {}), ("ab2", "mixed", 2000, dict(rings_per_thread=2, cluster_ctas=4)),
+    ("ab2", "mixed", 6000, dict(rings_per_thread=8, cluster_ctas=3)),
     ("ab2", "fp64", 300, {}), ("ab2", "fp64", 3000, {}), ("ab2", "fp64", 500, dict(block_threads=256)),
     ("ab2", "fp64", 500, dict(block_threads=64)),
     ("grid", "mixed", 1500, {}), ("grid", "mixed", 500, dict(block_threads=64, cluster_ctas=1)),
