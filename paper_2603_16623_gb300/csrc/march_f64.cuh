@@ -37,6 +37,7 @@
 // zero and whose matrix is the identity.
 #pragma once
 
+#include "f64_log.cuh"
 #include "march.cuh"
 #include "rank_sort.cuh"
 
@@ -59,36 +60,8 @@ __device__ __forceinline__ bool f64_finite(double x) {
 // a < b for radii (>= 0) on the integer pipe
 __device__ __forceinline__ bool f64_below(double a, double b) { return radius_key(a) < radius_key(b); }
 
-// The natural logarithm by a table of 128 reciprocals (the table-driven
-// method of P. T. P. Tang, ACM TOMS 16, 1990): x = 2^e m, c ~ 1/m from the
-// table, ln x = e ln 2 - ln c + log1p(m c - 1), the last by its series
-// (|m c - 1| < 2^-7.9: the first term left out is below 2^-58).  11 FP64
-// operations, where the library's log takes the pipe for 32 (2050 against
-// 700 cycles for a warp); absolute error below 2^-52 (1 + |ln x|).
-struct F64Log {
-    double c[128], lc[128];  // 1/m to 24 bits, and -ln of that
-    __device__ __forceinline__ void fill() {
-        for (int i = threadIdx.x; i < 128; i += blockDim.x) {
-            c[i] = (double)(1.0f / (1.0f + ((float)i + 0.5f) / 128.0f));
-            lc[i] = -log(c[i]);
-        }
-    }
-    __device__ __forceinline__ double operator()(double x) const {
-        const int hi = __double2hiint(x);
-        if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log(x);  // 0, subnormal, negative, inf, NaN
-        const int i = (hi >> 13) & 127;
-        const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(x));
-        // the exponent as a double without a conversion: 2^52 + 2^31 + e less 2^52 + 2^31
-        const double e = __hiloint2double(0x43300000, ((hi >> 20) - 1023) ^ (int)0x80000000) - 4503601774854144.0;
-        const double z = fma(m, c[i], -1.0);
-        double p = fma(-1.0 / 6.0, z, 0.2);
-        p = fma(p, z, -0.25);
-        p = fma(p, z, 1.0 / 3.0);
-        p = fma(p, z, -0.5);
-        const double y = fma(z * z, p, z);
-        return fma(e, 6.931471805599453094172e-01, lc[i]) + fma(e, 2.3190468138462995584e-17, y);
-    }
-};
+// the logarithm's table, copied to shared memory when a launch starts
+static __device__ const F64LogTable kF64LogTable = f64_log_table();
 
 // What the scans leave in shared memory: the warps' and the blocks' totals
 // and what one warp makes of them for the others; one per scan of a slice,
@@ -276,7 +249,7 @@ march_f64_kernel(const WakeDev<PrecF64>* __restrict__ wakes, const int32_t* __re
     __shared__ int64_t s_keys[64];
     __shared__ F64Sum2 s_w, s_g;
     __shared__ F64Mat s_m;
-    __shared__ F64Log s_log;
+    __shared__ F64LogTable s_log;
 
     const uint64_t t_launch = global_ns();
     WakeCtas C;
@@ -343,7 +316,8 @@ march_f64_kernel(const WakeDev<PrecF64>* __restrict__ wakes, const int32_t* __re
         W.rid[b][p] = id[k];
     };
     load();
-    s_log.fill();
+    for (int i = tid; i < 3 * kLogCells; i += T)
+        reinterpret_cast<double*>(&s_log)[i] = reinterpret_cast<const double*>(&kF64LogTable)[i];
     __syncthreads();
 
     // the beam offsets of this slice and the next, loaded one slice ahead
@@ -470,7 +444,7 @@ march_f64_kernel(const WakeDev<PrecF64>* __restrict__ wakes, const int32_t* __re
         double lnr[K], sw = 0.0, sl = 0.0;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            lnr[k] = k < np ? s_log(r[k]) : 0.0;
+            lnr[k] = k < np ? f64_log(s_log, r[k]) : 0.0;
             sw += w[k];
             sl = fma(w[k], lnr[k], sl);
         }
@@ -628,7 +602,7 @@ march_f64_kernel(const WakeDev<PrecF64>* __restrict__ wakes, const int32_t* __re
                 double psi_x, dprx, dpzx, bpx, bbx;
                 if (x > 0.0) {
                     const int k = lower_bound_dev(reinterpret_cast<const int64_t*>(sR), n, radius_key(x));
-                    const double ix = __drcp_rn(x), lnx = s_log(x), x2 = x * x;
+                    const double ix = __drcp_rn(x), lnx = f64_log(s_log, x), x2 = x * x;
                     const double Sk = W.regS[k];
                     const bool inside = x < rmax;
                     const double pion = x <= rmax ? c0 - x2 * quarter_n : Imax * -lnx;
