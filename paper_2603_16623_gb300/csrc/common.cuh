@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "ring_jump.cuh"  // (Mat2)
+
 namespace gbwake {
 
 // control words of a wake (device ints): next slice, status, failing
@@ -181,11 +183,7 @@ __device__ __forceinline__ Trip<T> shfl_idx_t(Trip<T> v, int l) {
     return {shfl_idx_t(v.x, l), shfl_idx_t(v.y, l), shfl_idx_t(v.c, l)};
 }
 
-// 2x2 matrix and the affine map x -> M x + c
-template <class R>
-struct Mat2 {
-    R m00, m01, m10, m11;
-};
+// the affine map x -> M x + c
 template <class R>
 struct Aff2 {
     R m00, m01, m10, m11, c0, c1;
@@ -240,6 +238,11 @@ struct OpMatLeft {
         return {b.m00 * a.m00 + b.m01 * a.m10, b.m00 * a.m01 + b.m01 * a.m11,
                 b.m10 * a.m00 + b.m11 * a.m10, b.m10 * a.m01 + b.m11 * a.m11};
     }
+    static constexpr bool kDev = false;  // (operands as they are: see OpMatDevLeft)
+    template <class R>
+    __device__ __forceinline__ static Mat2<R> one() { return {1, 0, 0, 1}; }
+    template <class R>
+    __device__ __forceinline__ static Mat2<R> whole(Mat2<R> m) { return m; }
 };
 // composition of affine maps, a applied first: x -> Mb (Ma x + ca) + cb
 struct OpAffThen {
@@ -464,16 +467,16 @@ struct SumMats {
     A t;
     Mat2<R> f, r;
 };
-template <bool TOT, class A, class R>
+template <bool TOT, class Op = OpMatLeft, class A, class R>
 __device__ __forceinline__ A block_excl_scan_sum_mats1(A t, Mat2<R> mf, Mat2<R> mr, A zero, SumMats<A, R>* sbuf,
                                                        Mat2<R>& ef, Mat2<R>& er, A& tt, Mat2<R>& tf, Mat2<R>& tr) {
-    const Mat2<R> I2 = {1, 0, 0, 1};
+    const Mat2<R> I2 = Op::template one<R>();
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int nw = blockDim.x >> 5;
     A it = warp_incl_scan<false>(t, OpAdd());
-    Mat2<R> ix = warp_incl_scan<false>(mf, OpMatLeft());
-    Mat2<R> iy = warp_incl_scan<true>(mr, OpMatLeft());
+    Mat2<R> ix = warp_incl_scan<false>(mf, Op());
+    Mat2<R> iy = warp_incl_scan<true>(mr, Op());
     A et = shfl_up_t(it, 1);
     Mat2<R> ex = shfl_up_t(ix, 1), ey = shfl_dn_t(iy, 1);
     if (lane == 0) {
@@ -495,8 +498,8 @@ __device__ __forceinline__ A block_excl_scan_sum_mats1(A t, Mat2<R> mf, Mat2<R> 
         wy = sbuf[lane].r;
     }
     A st = warp_incl_scan_n<false>(wt, OpAdd(), nw);
-    Mat2<R> sx = warp_incl_scan_n<false>(wx, OpMatLeft(), nw);
-    Mat2<R> sy = warp_incl_scan_n<true>(wy, OpMatLeft(), nw);
+    Mat2<R> sx = warp_incl_scan_n<false>(wx, Op(), nw);
+    Mat2<R> sy = warp_incl_scan_n<true>(wy, Op(), nw);
     const int last = scan_last_lane(nw);
     tt = shfl_idx_t(st, last);
     A qt = shfl_up_t(st, 1);
@@ -506,8 +509,8 @@ __device__ __forceinline__ A block_excl_scan_sum_mats1(A t, Mat2<R> mf, Mat2<R> 
         qx = I2;
     }
     if (lane == 31) qy = I2;
-    ef = OpMatLeft()(shfl_idx_t(qx, warp), ex);
-    er = OpMatLeft()(shfl_idx_t(qy, warp), ey);
+    ef = Op()(shfl_idx_t(qx, warp), ex);
+    er = Op()(shfl_idx_t(qy, warp), ey);
     if (TOT) {
         tf = shfl_idx_t(sx, last);
         tr = shfl_idx_t(sy, 0);

@@ -28,6 +28,8 @@
 // registers do not hold a thread's values (2 at 512 threads).
 #pragma once
 
+#include <type_traits>
+
 #include "march_rk4.cuh"
 #include "rank_sort.cuh"
 
@@ -103,8 +105,8 @@ __device__ __forceinline__ void ring_sources(R w, R r, R u, R pb, R g, R dpr, R 
 }
 
 // The jump matrices of a thread's rings multiplied up (Mf, later rings on the
-// left) and their inverses multiplied back (Mb); Ac: Eq. b_coeffs_1, m01 =
-// Ac / (2 r).
+// left) and their inverses multiplied back (Mb), as they are or less the
+// identity (Op, ring_jump.cuh); Ac: Eq. b_coeffs_1, m01 = Ac / (2 r).
 template <int K, class R>
 __device__ __forceinline__ Mat2<R> ring_matrix(R r, R Ac, R m01) {
     const R hA = (R)0.5 * Ac;
@@ -115,22 +117,28 @@ __device__ __forceinline__ Mat2<R> ring_inverse(R r, R Ac, R m01) {
     const R hA = (R)0.5 * Ac;
     return {(R)1 - hA * r, -m01, hA * r * r * r, (R)1 + hA * r};
 }
-template <int K, class R>
+template <int K, class Op = OpMatLeft, class R>
 __device__ __forceinline__ void ring_products(const R (&r)[K], const R (&Ac)[K], const R (&m01)[K], int np,
                                               Mat2<R>& Mf, Mat2<R>& Mb) {
-    Mf = Mb = {1, 0, 0, 1};
+    Mf = Mb = Op::template one<R>();
 #pragma unroll
     for (int k = 0; k < K; ++k)
-        if (k < np) Mf = OpMatLeft()(Mf, ring_matrix<K>(r[k], Ac[k], m01[k]));
+        if (k < np) {
+            if constexpr (Op::kDev) RingJump<R>(r[k], Ac[k], m01[k]).template multiply<false>(Mf);
+            else Mf = OpMatLeft()(Mf, ring_matrix<K>(r[k], Ac[k], m01[k]));
+        }
 #pragma unroll
     for (int k = K - 1; k >= 0; --k)
-        if (k < np) Mb = OpMatLeft()(Mb, ring_inverse<K>(r[k], Ac[k], m01[k]));
+        if (k < np) {
+            if constexpr (Op::kDev) RingJump<R>(r[k], Ac[k], m01[k]).template multiply<true>(Mb);
+            else Mb = OpMatLeft()(Mb, ring_inverse<K>(r[k], Ac[k], m01[k]));
+        }
 }
 
 // a8 from the exclusive products Yf, Yb: B^(p) at this thread's rings and
 // b_n; the regions' a, b to the tables where asked.  Takes an exchange and a
 // barrier over the wake, after which the tables are complete.
-template <class P, int K>
+template <class P, int K, class Op = OpMatLeft>
 __device__ __forceinline__ void gm_region_solve(const WakeDev<P>& W, WakeCtas& C, GmShared<P>& s, int n, int p0,
                                                 int np, const typename P::R (&r)[K], const typename P::R (&Ac)[K],
                                                 const typename P::R (&m01)[K], const typename P::R (&Bc)[K],
@@ -144,30 +152,40 @@ __device__ __forceinline__ void gm_region_solve(const WakeDev<P>& W, WakeCtas& C
     // R walked to the end of the rings
     R Ra[K], Rb[K];
     {
-        Mat2<R> Y = Yf;
+        Mat2<R> Y = Op::whole(Yf);
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            if (k < np) Y = OpMatLeft()(Y, ring_matrix<K>(r[k], Ac[k], m01[k]));
+            if (k < np) {
+                if constexpr (Op::kDev) RingJump<R>(r[k], Ac[k], m01[k]).cross(Y.m00, Y.m10);
+                else Y = OpMatLeft()(Y, ring_matrix<K>(r[k], Ac[k], m01[k]));
+            }
             Ra[k] = Y.m00;
             Rb[k] = Y.m10;
         }
     }
-    // R at the first region: as the thread before walked it
+    // R at the first region: its own product's, or as the thread before walked it
     const bool first = C.rank == 0 && tid == 0;
-    R q0 = shfl_up_t(Ra[K - 1], 1), q1 = shfl_up_t(Rb[K - 1], 1);
-    if (lane == 31) {
-        s.edge_r[0][warp] = Ra[K - 1];
-        s.edge_r[1][warp] = Rb[K - 1];
-    }
-    if (C.size > 1 && tid == (int)blockDim.x - 1) {  // for the next block
-        W.Ra[p0 + np] = Ra[K - 1];
-        W.Rb[p0 + np] = Rb[K - 1];
+    R q0, q1;
+    if constexpr (Op::kDev) {
+        q0 = Op::whole(Yf).m00;
+        q1 = Yf.m10;
+    } else {
+        q0 = shfl_up_t(Ra[K - 1], 1);
+        q1 = shfl_up_t(Rb[K - 1], 1);
+        if (lane == 31) {
+            s.edge_r[0][warp] = Ra[K - 1];
+            s.edge_r[1][warp] = Rb[K - 1];
+        }
+        if (C.size > 1 && tid == (int)blockDim.x - 1) {  // for the next block
+            W.Ra[p0 + np] = Ra[K - 1];
+            W.Rb[p0 + np] = Rb[K - 1];
+        }
     }
     // ---- the Green's sums, D walked back
     A gl = zeroA, dl = zeroA;
     R gp[K], dp[K], Da[K], Db[K];
     {
-        Mat2<R> Y = Yb;
+        Mat2<R> Y = Op::whole(Yb);
 #pragma unroll
         for (int k = K - 1; k >= 0; --k)
             if (k < np) {
@@ -179,7 +197,8 @@ __device__ __forceinline__ void gm_region_solve(const WakeDev<P>& W, WakeCtas& C
                 dp[k] = (Ra[k] * s1 - Rb[k] * s0) / wr;
                 gl = acc_add_r(gl, gp[k]);
                 dl = acc_add_r(dl, dp[k]);
-                Y = OpMatLeft()(Y, ring_inverse<K>(r[k], Ac[k], m01[k]));
+                if constexpr (Op::kDev) RingJump<R>(r[k], Ac[k], m01[k]).cross_back(Y.m01, Y.m11);
+                else Y = OpMatLeft()(Y, ring_inverse<K>(r[k], Ac[k], m01[k]));
                 Da[k] = Y.m01;
                 Db[k] = Y.m11;
             }
@@ -199,17 +218,19 @@ __device__ __forceinline__ void gm_region_solve(const WakeDev<P>& W, WakeCtas& C
         d_tot = s.tot_g.x;
     }
     // ---- a8: the regions' a, b
-    if (lane == 0 && warp > 0) {
-        q0 = s.edge_r[0][warp - 1];
-        q1 = s.edge_r[1][warp - 1];
-    }
-    if (tid == 0 && C.rank > 0 && np > 0) {
-        q0 = W.Ra[p0];
-        q1 = W.Rb[p0];
-    }
-    if (first) {
-        q0 = 1;
-        q1 = 0;
+    if constexpr (!Op::kDev) {
+        if (lane == 0 && warp > 0) {
+            q0 = s.edge_r[0][warp - 1];
+            q1 = s.edge_r[1][warp - 1];
+        }
+        if (tid == 0 && C.rank > 0 && np > 0) {
+            q0 = W.Ra[p0];
+            q1 = W.Rb[p0];
+        }
+        if (first) {
+            q0 = 1;
+            q1 = 0;
+        }
     }
     R ak[K], bk[K];
     {
@@ -277,7 +298,7 @@ __device__ __forceinline__ void gm_region_solve(const WakeDev<P>& W, WakeCtas& C
 // thread's K radii (r, rlo), momenta u, logarithms and weights, and B^(b).
 // `tables`: the region tables are written for the fields at other radii (they
 // are complete after the caller's next barrier over the wake).
-template <class P, int K>
+template <class P, int K, class Op = OpMatLeft>
 struct GmFields {
     using R = typename P::R;
     using A = typename P::A;
@@ -290,7 +311,7 @@ struct GmFields {
                                              const A (&wha)[K], const R (&bb)[K], bool tables) {
         const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
         const A zeroA = acc_zero(A());
-        const Mat2<R> I2 = {1, 0, 0, 1};
+        const Mat2<R> one = Op::template one<R>();
         // ---- a4
         Pair<A> loc = {zeroA, zeroA};
 #pragma unroll
@@ -342,25 +363,25 @@ struct GmFields {
                 m01[k] = (R)0.5 * Ac[k] / r[k];
             }
         Mat2<R> Mf, Mb;
-        ring_products<K>(r, Ac, m01, np, Mf, Mb);
+        ring_products<K, Op>(r, Ac, m01, np, Mf, Mb);
         A Ttot;
         Mat2<R> Yf, Yb, tf, tb;
-        A Tex = block_excl_scan_sum_mats1<true>(tl, Mf, Mb, zeroA, s.m, Yf, Yb, Ttot, tf, tb);
+        A Tex = block_excl_scan_sum_mats1<true, Op>(tl, Mf, Mb, zeroA, s.m, Yf, Yb, Ttot, tf, tb);
         if (C.size > 1) {
             const SumMats<A, R>* buf = C.exchange(SumMats<A, R>{Ttot, tf, tb});
             const int T = blockDim.x;
             Mat2<R> all;
             if (tid == 32 % T)
-                gm_fold<true>(C, buf, I2, OpMatLeft(), [](SumMats<A, R> v) { return v.r; }, s.pre_r, all);
+                gm_fold<true>(C, buf, one, Op(), [](SumMats<A, R> v) { return v.r; }, s.pre_r, all);
             if (tid == 64 % T)
                 gm_fold<false>(C, buf, zeroA, OpAdd(), [](SumMats<A, R> v) { return v.t; }, s.pre_t, s.tot_t);
             if (tid == 0)
-                gm_fold<false>(C, buf, I2, OpMatLeft(), [](SumMats<A, R> v) { return v.f; }, s.pre_f, all);
+                gm_fold<false>(C, buf, one, Op(), [](SumMats<A, R> v) { return v.f; }, s.pre_f, all);
             __syncthreads();
             Tex = acc_add(s.pre_t, Tex);
             Ttot = s.tot_t;
-            Yf = OpMatLeft()(s.pre_f, Yf);
-            Yb = OpMatLeft()(s.pre_r, Yb);
+            Yf = Op()(s.pre_f, Yf);
+            Yb = Op()(s.pre_r, Yb);
         }
 
         // ---- a6 + a7
@@ -384,7 +405,7 @@ struct GmFields {
             W.regT[n] = (R)0;
         }
         R bn;
-        gm_region_solve<P, K>(W, C, s, n, p0, np, r, Ac, m01, Bc, Cc, Yf, Yb, tables, bp, bn);
+        gm_region_solve<P, K, Op>(W, C, s, n, p0, np, r, Ac, m01, Bc, Cc, Yf, Yb, tables, bp, bn);
         // ---- guard
         bad = false;
 #pragma unroll
@@ -762,7 +783,9 @@ march_reg_kernel(const WakeDev<P>* __restrict__ wakes, const int32_t* __restrict
             }
         }
         // ---------------- a4..a8
-        GmFields<P, K> F;
+        // (matrices less the identity where their rounding shows: see ring_jump.cuh)
+        using Op = typename std::conditional<K >= 3 && std::is_same<P, PrecMixed>::value, OpMatDevLeft, OpMatLeft>::type;
+        GmFields<P, K, Op> F;
         F.evaluate(W, col, C, s_ev, n, p0, np, r, rlo, u, lnr, wa, wha, bb, tables);
         if (tables) stage_radii(W.rho[buf], n, sR);
         if (!query) F.dump(W, slice, n, np, id, r, u, bb);
