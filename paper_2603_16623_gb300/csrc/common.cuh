@@ -164,30 +164,6 @@ __device__ __forceinline__ Pair<T> shfl_dn_t(Pair<T> v, int o) { return {shfl_dn
 template <class T>
 __device__ __forceinline__ Pair<T> shfl_idx_t(Pair<T> v, int l) { return {shfl_idx_t(v.x, l), shfl_idx_t(v.y, l)}; }
 
-// two accumulators and an integer count scanned together
-template <class T>
-struct Trip {
-    T x, y;
-    int64_t c;
-};
-template <class T>
-__device__ __forceinline__ Trip<T> shfl_up_t(Trip<T> v, int o) {
-    return {shfl_up_t(v.x, o), shfl_up_t(v.y, o), shfl_up_t(v.c, o)};
-}
-template <class T>
-__device__ __forceinline__ Trip<T> shfl_dn_t(Trip<T> v, int o) {
-    return {shfl_dn_t(v.x, o), shfl_dn_t(v.y, o), shfl_dn_t(v.c, o)};
-}
-template <class T>
-__device__ __forceinline__ Trip<T> shfl_idx_t(Trip<T> v, int l) {
-    return {shfl_idx_t(v.x, l), shfl_idx_t(v.y, l), shfl_idx_t(v.c, l)};
-}
-
-// the affine map x -> M x + c
-template <class R>
-struct Aff2 {
-    R m00, m01, m10, m11, c0, c1;
-};
 template <class R>
 __device__ __forceinline__ Mat2<R> shfl_up_t(Mat2<R> v, int o) {
     return {shfl_up_t(v.m00, o), shfl_up_t(v.m01, o), shfl_up_t(v.m10, o), shfl_up_t(v.m11, o)};
@@ -200,17 +176,6 @@ template <class R>
 __device__ __forceinline__ Mat2<R> shfl_idx_t(Mat2<R> v, int l) {
     return {shfl_idx_t(v.m00, l), shfl_idx_t(v.m01, l), shfl_idx_t(v.m10, l), shfl_idx_t(v.m11, l)};
 }
-template <class R>
-__device__ __forceinline__ Aff2<R> shfl_up_t(Aff2<R> v, int o) {
-    return {shfl_up_t(v.m00, o), shfl_up_t(v.m01, o), shfl_up_t(v.m10, o),
-            shfl_up_t(v.m11, o), shfl_up_t(v.c0, o), shfl_up_t(v.c1, o)};
-}
-template <class R>
-__device__ __forceinline__ Aff2<R> shfl_dn_t(Aff2<R> v, int o) {
-    return {shfl_dn_t(v.m00, o), shfl_dn_t(v.m01, o), shfl_dn_t(v.m10, o),
-            shfl_dn_t(v.m11, o), shfl_dn_t(v.c0, o), shfl_dn_t(v.c1, o)};
-}
-
 // ---------------------------------------------------------------------------
 // operators: op(a, b) = "a, then b" where a covers the earlier elements of
 // the scan order
@@ -223,12 +188,6 @@ struct OpAddPair {
     template <class T>
     __device__ __forceinline__ Pair<T> operator()(Pair<T> a, Pair<T> b) const {
         return {acc_add(a.x, b.x), acc_add(a.y, b.y)};
-    }
-};
-struct OpAddTrip {
-    template <class T>
-    __device__ __forceinline__ Trip<T> operator()(Trip<T> a, Trip<T> b) const {
-        return {acc_add(a.x, b.x), acc_add(a.y, b.y), a.c + b.c};
     }
 };
 // matrix product, later element on the left: result = b * a
@@ -244,16 +203,6 @@ struct OpMatLeft {
     template <class R>
     __device__ __forceinline__ static Mat2<R> whole(Mat2<R> m) { return m; }
 };
-// composition of affine maps, a applied first: x -> Mb (Ma x + ca) + cb
-struct OpAffThen {
-    template <class R>
-    __device__ __forceinline__ Aff2<R> operator()(Aff2<R> a, Aff2<R> b) const {
-        return {b.m00 * a.m00 + b.m01 * a.m10, b.m00 * a.m01 + b.m01 * a.m11,
-                b.m10 * a.m00 + b.m11 * a.m10, b.m10 * a.m01 + b.m11 * a.m11,
-                b.m00 * a.c0 + b.m01 * a.c1 + b.c0, b.m10 * a.c0 + b.m11 * a.c1 + b.c1};
-    }
-};
-
 // ---------------------------------------------------------------------------
 // block-wide exclusive scan.  REV = false: thread order 0, 1, ...;
 // REV = true: the scan runs from the last thread down.  blockDim.x must be a
@@ -358,58 +307,7 @@ __device__ Pair<T> block_excl_scan_fwd_rev(T fx, T ry, T zero, Pair<T>* sbuf, T&
     return res;
 }
 
-// Forward product scan of mf and reverse product scan of mr in one pass
-// (op: later element on the left).  sbuf holds 33 Pair<Mat2<R>>.  With
-// TOT, tf and tr receive the block's forward and reverse products.
-template <bool TOT, class R>
-__device__ __forceinline__ void block_excl_scan_mat_fwd_rev_t(Mat2<R> mf, Mat2<R> mr, Pair<Mat2<R>>* sbuf,
-                                                              Mat2<R>& ef, Mat2<R>& er, Mat2<R>& tf, Mat2<R>& tr) {
-    const Mat2<R> I2 = {1, 0, 0, 1};
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int nw = blockDim.x >> 5;
-    Mat2<R> ix = warp_incl_scan<false>(mf, OpMatLeft());
-    Mat2<R> iy = warp_incl_scan<true>(mr, OpMatLeft());
-    Mat2<R> ex = shfl_up_t(ix, 1), ey = shfl_dn_t(iy, 1);
-    if (lane == 0) ex = I2;
-    if (lane == 31) ey = I2;
-    if (lane == 31) sbuf[warp].x = ix;
-    if (lane == 0) sbuf[warp].y = iy;
-    __syncthreads();
-    if (warp == 0) {
-        Mat2<R> wx = lane < nw ? sbuf[lane].x : I2;
-        Mat2<R> wy = lane < nw ? sbuf[lane].y : I2;
-        Mat2<R> sx = warp_incl_scan<false>(wx, OpMatLeft());
-        Mat2<R> sy = warp_incl_scan<true>(wy, OpMatLeft());
-        Mat2<R> qx = shfl_up_t(sx, 1), qy = shfl_dn_t(sy, 1);
-        if (lane == 0) qx = I2;
-        if (lane == 31) qy = I2;
-        __syncwarp();
-        if (lane < nw) {
-            sbuf[lane].x = qx;
-            sbuf[lane].y = qy;
-        }
-        if (lane == 31) sbuf[32].x = sx;
-        if (lane == 0) sbuf[32].y = sy;
-    }
-    __syncthreads();
-    ef = OpMatLeft()(sbuf[warp].x, ex);
-    er = OpMatLeft()(sbuf[warp].y, ey);
-    if (TOT) {
-        tf = sbuf[32].x;
-        tr = sbuf[32].y;
-    }
-    __syncthreads();
-}
-
-template <class R>
-__device__ void block_excl_scan_mat_fwd_rev(Mat2<R> mf, Mat2<R> mr, Pair<Mat2<R>>* sbuf, Mat2<R>& ef,
-                                            Mat2<R>& er) {
-    Mat2<R> tf, tr;
-    block_excl_scan_mat_fwd_rev_t<false>(mf, mr, sbuf, ef, er, tf, tr);
-}
-
-// One-barrier forms of the three block scans above, with the same
+// One-barrier forms of the two block scans above, with the same
 // arithmetic in the same order (bitwise the same results): every warp scans
 // the warp totals itself instead of warp 0 scanning them between two more
 // barriers.  sbuf needs nw (not 33) values; every warp reads it after the

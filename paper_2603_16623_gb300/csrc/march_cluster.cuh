@@ -86,7 +86,7 @@ __device__ __forceinline__ void fold_rev(const T* recv, int rank, int size, T id
     }
 }
 
-// The same folds by thread 0 into shared memory, read by every thread after
+// The forward fold by thread 0 into shared memory, read by every thread after
 // a block barrier (keeps the fold's registers out of the callers' peak).
 template <class T, class Op>
 __device__ __forceinline__ void fold_fwd_shared(const T* recv, int rank, int size, T ident, Op op, T* s_pre,
@@ -94,18 +94,6 @@ __device__ __forceinline__ void fold_fwd_shared(const T* recv, int rank, int siz
     if (threadIdx.x == 0) {
         T pre, all;
         fold_fwd(recv, rank, size, ident, op, pre, all);
-        *s_pre = pre;
-        *s_all = all;
-    }
-    __syncthreads();
-}
-
-template <class T, class Op>
-__device__ __forceinline__ void fold_rev_shared(const T* recv, int rank, int size, T ident, Op op, T* s_pre,
-                                                T* s_all) {
-    if (threadIdx.x == 0) {
-        T pre, all;
-        fold_rev(recv, rank, size, ident, op, pre, all);
         *s_pre = pre;
         *s_all = all;
     }
@@ -853,9 +841,9 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
             const float lo_r = crank > 0 ? s_last[crank - 1] : -INFINITY;
             const float hi_r = last_cta ? INFINITY : s_last[crank];
             if (mode == MODE_MARCH) {
-                // the particles split as in a3 (own range, or an even share
-                // of the slice with the owner's tables read remotely);
-                // region k (radii in (rho_{k-1}, rho_k]) lives in the CTA
+                // the particles of this CTA's own range, or (more of them than
+                // threads) an even share of the slice with the owner's
+                // tables read remotely; region k (radii in (rho_{k-1}, rho_k]) lives in the CTA
                 // holding ring k, region n in the last CTA
                 const int mc = dist ? (m + csize - 1) / csize : m;
                 const int c0q = dist ? crank * mc : 0;
@@ -896,7 +884,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                     }
                     R psi, dpr, dpz, bp, bb = 0.f;
                     if (x > 0.f) {
-                        kr = kr < 0 ? ring_rank_all<K>(so.rh, nl_o, x) : ring_rank_from<K>(so.rh, nl_o, kr, x, true);
+                        kr = kr < 0 ? ring_rank_all<K>(so.rh, nl_o, x) : ring_rank_from<K>(so.rh, nl_o, kr, x);
                         fast_fields_region<K>(so, nl_o, TK, kr, x, rmax, half_n, quarter_n, Wtot, Imax, c0, &dpr,
                                               &dpz, &bp, &psi);
                         bb = qb_s[j] * inv_2pi_dxi / x;
@@ -925,7 +913,7 @@ march_cluster_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t
                     if (!(x > lo_r && x <= hi_r) && !(crank == 0 && x != x)) continue;
                     R psi, dpr, dpz, bp, bb = 0.f;
                     if (x > 0.f) {
-                        const int kl = ring_rank<K>(sm.rh, nl, x, true);
+                        const int kl = ring_rank<K>(sm.rh, nl, x);
                         fast_fields_region<K>(sm, nl, TK, kl, x, rmax, half_n, quarter_n, Wtot, Imax, c0, &dpr,
                                               &dpz, &bp, &psi);
                         if (m > 0) {

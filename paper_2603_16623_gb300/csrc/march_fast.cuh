@@ -211,21 +211,21 @@ __device__ __forceinline__ void resort(const FastSmem& sm, int n, int& skip) {
     }
 }
 
-// number of sorted rings with radius < x (strict) or <= x
+// number of sorted rings with radius < x
 template <int K>
-__device__ __forceinline__ int ring_rank(const float* rh, int n, float x, bool strict) {
+__device__ __forceinline__ int ring_rank(const float* rh, int n, float x) {
     using SW = Swz<K>;
     int lo = 0, hi = n;
     while (lo < hi) {
         int mid = (lo + hi) >> 1;
         float v = rh[SW::at(mid)];
-        if (strict ? (v < x) : (v <= x)) lo = mid + 1;
+        if (v < x) lo = mid + 1;
         else hi = mid;
     }
     return lo;
 }
 
-// The same, strict, in a fixed number of steps (the threads of a warp stay together).
+// The same in a fixed number of steps (the threads of a warp stay together).
 template <int K>
 __device__ __forceinline__ int ring_rank_all(const float* rh, int n, float x) {
     using SW = Swz<K>;
@@ -238,18 +238,15 @@ __device__ __forceinline__ int ring_rank_all(const float* rh, int n, float x) {
     return lo;
 }
 
-// Rank of x among the sorted radii rh[0, n) (how many are < x, or <= x when
-// !strict), given a rank `from` that does not exceed it: galloping from
-// `from` (steps 1, 2, 4, ...), then a binary search inside the last step.
+// Rank of x among the sorted radii rh[0, n) (how many are < x), given a rank
+// `from` that does not exceed it: galloping from `from` (steps 1, 2, 4, ...),
+// then a binary search inside the last step.
 // Along a run of increasing radii successive ranks are close, so this costs
 // O(log distance) instead of O(log n).
 template <int K>
-__device__ __forceinline__ int ring_rank_from(const float* rh, int n, int from, float x, bool strict) {
+__device__ __forceinline__ int ring_rank_from(const float* rh, int n, int from, float x) {
     using SW = Swz<K>;
-    auto below = [&](int i) {
-        const float v = rh[SW::at(i)];
-        return strict ? (v < x) : (v <= x);
-    };
+    auto below = [&](int i) { return rh[SW::at(i)] < x; };
     if (from >= n || !below(from)) return from;
     int lo = from, step = 1;  // invariant: below(lo)
     int hi = lo + 1;
@@ -308,7 +305,7 @@ template <int K>
 __device__ __forceinline__ void fast_fields_at(const FastSmem& sm, int n, int TK, float x, float rmax, float half_n,
                                                float quarter_n, ff Wtot, ff Imax, ff c0, float* dpr, float* dpz,
                                                float* bp, float* psi) {
-    const int k = ring_rank<K>(sm.rh, n, x, true);
+    const int k = ring_rank<K>(sm.rh, n, x);
     fast_fields_region<K>(sm, n, TK, k, x, rmax, half_n, quarter_n, Wtot, Imax, c0, dpr, dpz, bp, psi);
 }
 
@@ -825,7 +822,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
 
         // ---------------- a9: fields on the beam particles (or query radii)
         if (mode == MODE_MARCH) {
-            // contiguous runs of the radius-sorted particles, as in a3
+            // contiguous runs of the radius-sorted particles
             const int per = (m + T - 1) / T;
             const int q1 = min(m, (tid + 1) * per);
             int kr = -1;  // (the first particle searches all rings, the next go on from there)
@@ -843,7 +840,7 @@ march_fast_kernel(const WakeDev<PrecMixed>* __restrict__ wakes, const int32_t* _
                 const R x = xb[j];
                 R psi, dpr, dpz, bp, bb = 0.f;
                 if (x > 0.f) {
-                    kr = kr < 0 ? ring_rank_all<K>(sm.rh, n, x) : ring_rank_from<K>(sm.rh, n, kr, x, true);
+                    kr = kr < 0 ? ring_rank_all<K>(sm.rh, n, x) : ring_rank_from<K>(sm.rh, n, kr, x);
                     fast_fields_region<K>(sm, n, TK, kr, x, rmax, half_n, quarter_n, Wtot, Imax, c0, &dpr, &dpz,
                                           &bp, &psi);
                     bb = qb_s[j] * inv_2pi_dxi / x;
