@@ -419,7 +419,7 @@ def run_ours(args):
             "roofline": roofline, "cpu_baseline": cpu, "plain_fp64": plain,
             "beam_push": push, "beam_stage": stage_ab,
             "mobile_ions": _ions_roofline(ions, peak_tflops, sm_mhz),
-            "rk4": _alu_roofline(rk4, peak_tflops, sm_mhz, FLOPS_PER_RING_SLICE_RK4, "march_rk4_kernel<PrecMixed>", 1),
+            "rk4": _alu_roofline(rk4, peak_tflops, sm_mhz, FLOPS_PER_RING_SLICE_RK4, "march_rk4_reg_kernel<PrecMixed>", 1),
             "beam_grid": grid,
             "single_wakes": singles,
             "clocks": clocks,
@@ -585,15 +585,15 @@ def grid_bench(args, wakes, stream):
     """The paper's grid coupling (adaptive beam grids of 32 radial cells per
     beam) against the gridless one on the same batched wakes of <= 8192
     rings over a bounded window (their first args.grid_slices slices):
-    FP64 on the global-memory march, both on one block per wake (the grid's
-    own cost), and the grids on their automatic clusters; mixed, the grids
+    FP64, the grids on one block per wake and on their automatic clusters,
+    gridless on the on-chip march's; mixed, the grids
     on their automatic clusters against the gridless on-chip march; batched
     reset + step, CUDA-event timed."""
     import torch
     from paper_2603_16623_gb300 import wake as wm
     sel = [wk for wk in wakes if wk.n_rings <= 8192][: args.grid_wakes]
     out = {"wakes": len(sel), "slices": args.grid_slices, "grid_nr": 32,
-           "note": "fp64: gridless and grid on one block per wake, grid_clusters on the automatic clusters; "
+           "note": "fp64: grid on one block per wake, grid_clusters on the automatic clusters, gridless on the on-chip march; "
                    "mixed: grids on the automatic clusters, gridless on the on-chip march"}
     # (name, grid cells, precision, blocks per wake: 1, or 0 = automatic)
     for name, nr, prec, cl in (("gridless", 0, "fp64", 0), ("grid", 32, "fp64", 1), ("grid_clusters", 32, "fp64", 0),
@@ -666,7 +666,7 @@ def _ions_roofline(ions, peak_tflops, sm_mhz):
         return None
     achieved = FLOPS_PER_RING_SLICE_IONS * ions["ring_slices"] / (ions["march_ms"] / 1e3) / 1e12
     ions["roofline"] = {"bound": "alu", "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
-                        "frac": achieved / peak_tflops, "traffic": None, "kernel": "march_ions_kernel<PrecMixed>",
+                        "frac": achieved / peak_tflops, "traffic": None, "kernel": "march_ions_reg_kernel<PrecMixed>",
                         "flops_per_ring_slice": FLOPS_PER_RING_SLICE_IONS,
                         "peak_basis": "measured: FP32 FMA throughput microbenchmark (wake_measure_peaks)"}
     return ions

@@ -61,12 +61,13 @@ enum {
                       names: four field evaluations per slice, the beam source at
                       the half step the mean of the two slices; a stage state
                       below the axis is evaluated mirrored.  Electron-only wakes
-                      (no mobile ions) of at most 16384 rings, on the global-
-                      memory march: one block per wake, or a thread-block
-                      cluster of cluster_ctas (1..8) blocks that split the
-                      sorted rings (block 0 sorts the state and the stage
-                      states); 0 = automatic, the fewest blocks (at most 8)
-                      that hold at most 2 rings per thread.  rings_per_thread
+                      (no mobile ions) of at most 16384 rings: one block per
+                      wake, or a thread-block cluster of cluster_ctas (1..8)
+                      blocks that split the sorted rings; 0 = automatic, the
+                      fewest blocks (at most 8) that hold at most 2 rings per
+                      thread.  Up to 4 rings per thread (2 with more than 256
+                      threads; automatic: up to 8192 rings) they stay in
+                      registers, else in global memory.  rings_per_thread
                       must be 0. */
 };
 
@@ -153,7 +154,8 @@ typedef struct {
                                  with beam grids).  FP64 without these: 0 =
                                  the on-chip march (blocks of up to 128
                                  threads, up to 16 of them by the ring
-                                 count), else one block of that many threads */
+                                 count, wake_get_launch_config), else one
+                                 block of that many threads */
     int32_t rings_per_thread; /* MIXED: 2, 4 or 8 rings per thread; 0 = auto  */
     int32_t cluster_ctas;     /* MIXED: CTAs per wake, 1..16 (> 1: a thread-
                                  block cluster); 0 = automatic.  The threads
@@ -179,8 +181,8 @@ typedef struct {
                                  or a thread-block cluster (cluster_ctas
                                  0..8; 0 = automatic: the fewest blocks, at
                                  most 8, that hold at most 4 rings per
-                                 thread); block 0 sorts the rings and sums
-                                 the node charges. */
+                                 thread: in registers up to 8192 rings, in
+                                 global memory beyond). */
     double grid_rmax;         /* with grid_nr > 0: 0 = adaptive extents; > 0 =
                                  every grid spans [0, grid_rmax] (the regular
                                  intermediate grid).  Every beam particle must
@@ -248,6 +250,10 @@ wake_status wake_step_slices(wake_handle *h, int32_t n_slices);
    its particles); with mobile ions, the sums of both species.
    r and the outputs are host arrays (device_ptrs = 0) or device arrays
    (device_ptrs = 1); outputs are "real"; any output may be NULL.
+   Wakes of the mixed on-chip march (no ions, RK4 or grids) spread the radii
+   over as many blocks (or clusters) as they fill, up to one per SM, each of
+   which solves the slice: the shortest call alone, but beside work on other
+   streams up to 152 blocks of one slice each.
    Errors: EINVAL (n < 0, or the window is finished: no slice is left to
    sample), ENONFINITE (the wake stopped), ECUDA. */
 wake_status wake_fields_at(wake_handle *h, int64_t n, const double *r, void *ez, void *wr,
@@ -457,9 +463,8 @@ int64_t wake_max_slice_particles(int32_t precision); /* beam particles per slice
    predicted march time is at least wake_get_latency_shape_ms(), the latency
    shape (wake_launch_shape_latency).  n_steps 0: the batch shape.  Outputs
    (each may be NULL): threads per CTA, rings per thread and CTAs per wake
-   (> 1: a thread-block cluster); all three 0 when the wake runs on a
-   one-CTA march instead (FP64, or the automatic shape beyond the on-chip
-   march's 65,536 rings).  The launch-shape autotuner enumerates its
+   (> 1: a thread-block cluster); all three 0 with FP64, whose wakes have
+   no shape to choose here (wake_get_launch_config reports theirs).  The launch-shape autotuner enumerates its
    candidates with it.  Errors: EINVAL for a precision other than WAKE_FP64
    or WAKE_MIXED, n_rings outside [1, wake_max_rings(precision)], a negative
    n_steps, or the shape wake_init would refuse (rings_per_thread not 0, 2,
@@ -494,7 +499,7 @@ wake_status wake_launch_shape_latency(int32_t precision, int32_t n_rings, int32_
 wake_status wake_set_latency_shape_ms(double ms);
 double wake_get_latency_shape_ms(void);
 
-/* the global-memory marches whose wakes also run on thread-block clusters */
+/* the marches with a block size and a thread-block cluster to choose */
 enum { WAKE_GM_IONS = 1, WAKE_GM_RK4 = 2, WAKE_GM_GRID = 3 };
 
 /* The launch shape wake_init gives a wake of the two-species march

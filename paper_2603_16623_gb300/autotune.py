@@ -11,10 +11,14 @@ fills the GPU with copies of it (about `fill` x the SM count in CTAs, as a
 large batch does), times one batched march per candidate shape with CUDA
 events and keeps the fastest in ring-slices per second.  The automatic
 shape stays unless a candidate beats it by `min_gain`, so timing noise does
-not churn the table.  The global-memory marches (FP64, mobile ions, RK4,
-beam grids) are tuned the same way over their block size (block_threads),
-and those with mobile ions, RK4 or beam grids also over their blocks per
-wake (a thread-block cluster of 2, 4 or 8 blocks of the default size).
+not churn the table.  FP64 wakes and those with mobile ions, RK4 or beam
+grids are tuned the same way over their block size (block_threads), and
+these three also over their blocks per wake (a thread-block cluster of 2, 4
+or 8 blocks of the default size).  An FP64 wake's automatic shape is the
+on-chip march on up to 16 blocks, a block size the march in one block: on a
+GPU filled with wakes of 500 to 8000 rings the automatic one measured 1.3-1.8e9
+ring-slices/s and the best block size 1.1-1.2e9, alone 3 to 20 times as much,
+so a table's FP64 entry from before the on-chip march is better dropped.
 
 The candidates come from the library itself (wake_launch_shape: the shape
 wake_init would give, computed on the host), so the tuner never proposes a
@@ -38,14 +42,15 @@ from typing import Callable, Dict, List, Optional, Sequence
 from . import wake as wm
 from . import workloads as W
 
-# the kinds of march a table entry applies to: the on-chip march (mixed,
-# electrons over the ion column) and the global-memory marches
+# the kinds of march a table entry applies to: the mixed on-chip march
+# (electrons over the ion column) and those that take a block size
 KINDS = ("mixed", "fp64", "ions", "rk4", "grid")
 BLOCK_THREADS = (64, 128, 256, 512)
-# the block size wake_init takes when block_threads is 0 (timed as the
-# automatic candidate, so not again as an explicit one)
+# the block size left out of the explicit candidates: what wake_init takes
+# when block_threads is 0 (timed as the automatic candidate); with FP64, where
+# 0 is the on-chip march, 256 threads (never the fastest: measured above)
 DEFAULT_BLOCK_THREADS = {"fp64": 256, "grid": 256, "ions": 512, "rk4": 512}
-# the global-memory marches that also run as thread-block clusters
+# the kinds that also take thread-block clusters of blocks of that size
 GM_CLUSTER_KINDS = ("ions", "rk4", "grid")
 DEFAULT_SIZES = (512, 1024, 2048, 3072, 4096, 6144, 8192, 12288, 16384, 32768, 65536)
 
@@ -56,7 +61,7 @@ class Candidate:
     to for the size they were made for."""
     rings_per_thread: int = 0   # on-chip march: 0 (automatic), 2, 4 or 8
     cluster_ctas: int = 0       # on-chip march: 0 (automatic) or 1-16; ions, RK4, grids: 0 or 1-8
-    block_threads: int = 0      # global-memory marches: 0 (the library's default) or 64-512
+    block_threads: int = 0      # FP64, ions, RK4, grids: 0 (the library's choice) or 64-512
     threads: int = 0            # resolved threads per CTA (on-chip march)
     ctas: int = 1               # resolved CTAs per wake
 
@@ -79,7 +84,7 @@ def max_rings(kind: str) -> int:
         return wm.wake_max_rings("mixed")
     if kind == "ions":
         return 4096  # cells per species with mobile ions
-    return wm.wake_max_rings("fp64")  # the other global-memory marches: 8192 rings
+    return wm.wake_max_rings("fp64")  # FP64, RK4, grids: 8192 rings
 
 
 def candidates(n_rings: int, kind: str = "mixed", max_candidates: int = 8,
@@ -87,7 +92,7 @@ def candidates(n_rings: int, kind: str = "mixed", max_candidates: int = 8,
     """The shapes worth timing for a wake of n_rings rings: the automatic
     one first, then (on-chip march) every valid (rings per thread, CTAs per
     wake) with at least min_threads threads per CTA, thinned evenly to
-    max_candidates; or (global-memory marches) the block sizes 64-512 and,
+    max_candidates; or (FP64, ions, RK4, grids) the block sizes 64-512 and,
     with mobile ions, RK4 or beam grids, clusters of 2, 4 and 8 blocks of
     the default size."""
     if not 1 <= n_rings <= max_rings(kind):

@@ -228,7 +228,7 @@ __device__ __forceinline__ double make_radius(double hi, double) { return hi; }
 __device__ __forceinline__ ff make_radius(float hi, float lo) { return ff{hi, lo}; }
 
 // ring id's weight and self weight in the accumulator type: the mixed path
-// takes them float-float from the per-ring table ({w, what} = ctab[3 id + 1]),
+// takes them float-float from the per-ring table (RingTab's second part),
 // since their sum meets the exact ion column and FP32-rounded weights would
 // leave ~1e-7 of the enclosed charge
 __device__ __forceinline__ void ring_weights(const RingTab&, const double* w, const double* wh, int id, double& wa,

@@ -20,7 +20,7 @@
 //     integer pipe), and what a scan needs once per block is computed by one
 //     warp instead of by every thread.
 // Measured on GB300: one wake of 2000 rings 283 -> 26 us per slice; 24 wakes
-// of 500-8000 rings in one launch 1013 -> 68 us per slice.  What is left is
+// of 500-8000 rings in one batch 1013 -> 60 us per slice.  What is left is
 // the chain of ~350 FP64 instructions of one warp (a third of them the two
 // matrix scans) and five cluster barriers.
 // The suffix products of the decaying solution are formed as such (not as

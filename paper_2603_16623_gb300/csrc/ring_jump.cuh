@@ -8,17 +8,22 @@
 // of what the compiler fuses.  Here the matrices are multiplied less the
 // identity and the solutions walked across a ring by what it adds to them, so
 // that errors are relative to the difference.  The mixed march of beam-grid
-// wakes (march_reg_kernel) takes its products so at 3 and 4 rings per thread,
-// where they had lost precision against the global-memory march's: E_z
-// against 64 bits, over 20 solves with wakes of more than 4096 rings, median
-// 1.1e-6 -> 2.2e-7 and largest 1.9e-6 -> 6.7e-7 (the global-memory march
-// 4.2e-7 and 1.3e-6), B_theta 2.5e-7 -> 1.4e-7 (2.8e-7).  12 operations for a
-// product of two, where the matrices as they are take 8, and no exchange of R
-// between threads: 24 wakes 9.86 -> 9.92 ms.
-// The other marches keep the matrices as they are: over 24 to 40 solves each
-// their errors are those of the global-memory marches (ions, RK4, both
-// precisions, and FP64 AB2), FP64 wakes would be 6 % slower on their pipe, and
-// where rings cross another rounding moves the fields of single particles.
+// wakes (march_reg_kernel) takes its products so at 3 and 4 rings per thread
+// (its automatic shapes above 512 rings): with the matrices as they are it had
+// lost precision against the global-memory march above 4096 rings.  E_z
+// against 64 bits there, over 20 solves, median 1.1e-6 -> 2.2e-7 and largest
+// 1.9e-6 -> 6.7e-7 (the global-memory march 4.2e-7 and 1.3e-6), B_theta
+// 2.5e-7 -> 1.4e-7 (2.8e-7).  12 operations for a product of two, where the
+// matrices as they are take 8, and no exchange of R between threads: 24 wakes
+// 9.86 -> 9.92 ms (10.08 with this form above 4096 rings only: two kernels'
+// instructions to fetch instead of one's).
+// The other marches keep the matrices as they are.  FP64 (AB2, ions, RK4): the
+// errors are those of the global-memory marches, and 12 FP64 operations for 8
+// take 6 % on their pipe.  Mixed ions and RK4: E_z's error is 0.97 to 1.0 of
+// the global-memory marches' up to 2048 rings, 1.7 from there to 4096 and 0.9
+// above (RK4); this form brings 0.6 over all, but in their scans rings cross,
+// both are 4e-4 from 64 bits, and any other rounding moves single particles'
+// fields by 1e-2 to 1e-1: the results stay what they are.
 // Compiles for the host too (tests).
 #pragma once
 

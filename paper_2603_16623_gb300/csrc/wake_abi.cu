@@ -47,18 +47,22 @@ wake_status fail(wake_status st, const char* fmt, ...) {
                         __FILE__, __LINE__);                                                   \
     } while (0)
 
-constexpr int32_t kMaxRings = 8192;           // FP64 path (one CTA per wake, sort in shared memory)
+constexpr int32_t kMaxRings = 8192;           // FP64 AB2 wakes: 16 blocks of 128 threads x 4 rings, or one
+                                              // block whose shared memory sorts them
 constexpr int32_t kMaxIonCells = 4096;        // mobile ions: rings per species (2 x 4096 rings per wake)
-// the global-memory marches with mobile ions, RK4 or beam grids on thread-
-// block clusters: the automatic cluster's positions per thread (of each
-// species with ions), and a cluster's barriers per slice (per stage with
-// RK4), us
+// the marches with mobile ions, RK4 or beam grids on thread-block clusters:
+// the automatic cluster's positions per thread (of each species with ions),
+// and a cluster's barriers per slice (per stage with RK4), us.  All four are
+// fits to the marches with state in global memory; the register marches,
+// which serve these shapes up to 8192 rings (8 blocks at most), were not
+// timed at others.
 constexpr int32_t kIonRingsPerThread = 2;
 constexpr int32_t kRk4RingsPerThread = 2;
 constexpr int32_t kGridRingsPerThread = 4;
 constexpr double kGmClusterSliceUs = 20.0;
 constexpr int32_t kMaxRingsMixed = 65536;     // mixed path: a 16-CTA cluster of 512 threads x 8 rings
-constexpr int32_t kMaxRk4Rings = 16384;       // RK4, beam grids: the sort of one block (8 B per ring)
+constexpr int32_t kMaxRk4Rings = 16384;       // RK4, beam grids: the sort of one block (8 B per ring) in the
+                                              // marches that serve the wakes too wide for the registers
 constexpr int32_t kMaxSliceParticles = 8192;
 constexpr int32_t kDefaultThreads = 256;
 
@@ -684,7 +688,9 @@ cudaError_t launch_gm_reg(const wake_handle* h, const WakeDev<P>* d_wakes, const
 // block a thread's radii followed each other: 20,000 radii of a 2000-ring
 // wake 257 -> 62 us a call (of these the slice ~20, launch and wait ~15; the
 // descriptor from the pool instead of cudaMalloc and cudaFree ~100 of the
-// difference: 100 radii took 180).
+// difference: 100 radii took 180).  That is for a caller alone: beside a
+// batch on other streams the copies take SM time from it (about one slice
+// per block, the radii's own work being the same).
 int32_t query_copies(int32_t threads, int32_t cl, int64_t nq) {
     constexpr int64_t kSms = 152;
     return (int32_t)std::max<int64_t>(1, std::min((nq + threads - 1) / threads, kSms / cl));
@@ -945,14 +951,17 @@ wake_status batch_bucket(const std::vector<wake_handle*>& hs, const FastShape& s
 // on-chip march in shape f (threads > 0) or of a one-CTA kernel in blocks of
 // `threads` (per_thread rings each); the batch's plan only needs it to rank
 // wakes, wake_init to compare a wake with the latency-shape threshold.
-// Fitted to march times measured one wake at a time (wake_get_march_times):
-// at 4 rings per thread one CTA of R rings ~ 11 + 9 R/2048 us per slice and
-// a cluster of cl CTAs of R rings each ~ 16.3 + 1.6 cl + 8.9 R/1024 us (its
+// Fitted to march times measured one wake at a time (wake_get_march_times)
+// before the slices were shortened (a cluster of 6 blocks of 1024 rings: 34.8
+// us by the fit, 23.0 measured now), of which the order of the shapes is used:
+// at 4 rings per thread one CTA of R rings ~ 11 + 9 R/2048 us per slice and a
+// cluster of cl CTAs of R rings each ~ 16.3 + 1.6 cl + 8.9 R/1024 us (its
 // cluster barriers and exchanges), on the batched wakes; at 2 rings per
 // thread, from uniform wakes scaled by the batched wakes' 1.2x, one CTA
 // ~ 0.875 of the 4-ring time and a cluster ~ 17.8 + 0.26 cl + 6.4 R/1024 us.
-// The one-CTA kernels with state in global memory grow with the rings per
-// thread.
+// (The latency-shape threshold, off by default, compares these milliseconds.)
+// The two-species, RK4 and beam-grid marches are ranked by the fit to those
+// with state in global memory, which grow with the rings per thread.
 double predicted_fast_slice_us(const FastShape& f) {
     const double R = (double)f.threads * f.k;
     if (f.k == 2) return f.cl > 1 ? 17.8 + 0.26 * f.cl + 6.4 * R / 1024.0 : 0.875 * (11.0 + 9.0 * R / 2048.0);
@@ -1487,8 +1496,8 @@ wake_status wake_init(const wake_config* cfg, const wake_plasma_desc* plasma, co
         return fail(WAKE_EINVAL, "wake_init: RK4 wakes have at most %d rings (block 0 sorts the stage states in its "
                                  "shared memory)", kMaxRk4Rings);
     if (rk4 && (ions || cfg->rings_per_thread || cfg->cluster_ctas < 0 || cfg->cluster_ctas > kMaxWakeCtas))
-        return fail(WAKE_EINVAL, "wake_init: RK4 runs electron-only wakes on the global-memory march (no mobile "
-                                 "ions, rings_per_thread 0, cluster_ctas in [0, %d])", kMaxWakeCtas);
+        return fail(WAKE_EINVAL, "wake_init: RK4 runs electron-only wakes (no mobile ions, rings_per_thread 0, "
+                                 "cluster_ctas in [0, %d])", kMaxWakeCtas);
     if (cfg->grid_nr < 0 || cfg->grid_nr > 1024) return fail(WAKE_EINVAL, "wake_init: grid_nr must be in [0, 1024]");
     if (cfg->grid_nr > 0 && (cfg->rings_per_thread || cfg->cluster_ctas < 0 || cfg->cluster_ctas > kMaxWakeCtas))
         return fail(WAKE_EINVAL, "wake_init: beam-grid wakes take rings_per_thread 0 and cluster_ctas in [0, %d]",
@@ -1507,7 +1516,7 @@ wake_status wake_init(const wake_config* cfg, const wake_plasma_desc* plasma, co
     if (cfg->grid_nr > 0 && (rk4 || ions || n_beams > kMaxGridSpecies))
         return fail(WAKE_EINVAL, "wake_init: beam grids run WAKE_AB2, without mobile ions, with at most %d beam "
                                  "species", kMaxGridSpecies);
-    // the two-species and RK4 marches: one CTA of 512 threads per wake
+    // the two-species and RK4 marches: blocks of 512 threads
     if ((ions || rk4) && !cfg->block_threads) threads = 512;
     if (!plasma->r_edges) return fail(WAKE_EINVAL, "wake_init: r_edges is NULL");
     if (!(plasma->density > 0.0) || !std::isfinite(plasma->density))
