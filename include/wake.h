@@ -359,6 +359,9 @@ wake_status wake_get_ring_state(wake_handle *h, double *rho, double *ur, double 
    n_steps) with the given ring state by ring index (double host arrays of
    n_rings; rho >= 0).  f_rho and f_ur are the AB2 history; pass both NULL
    to start the next step with forward Euler.  Clears the stopped status.
+   rho and u_r must be finite; a history that is not, or overflows the
+   wake's real type, stops the wake (WAKE_ENONFINITE) at the slice after the
+   push that takes it.
    Errors: EINVAL, ENOMEM, ECUDA. */
 wake_status wake_set_ring_state(wake_handle *h, int32_t slice, const double *rho, const double *ur,
                                 const double *f_rho, const double *f_ur);

@@ -14,8 +14,9 @@
 //     sums of w and w ln rho; the d_zeta psi sum with the solve's matrices
 //     (both depend on psi only); the Green's sums;
 //   - two neighbours' edges: the regular solution walked to the end of the
-//     rings before (R at its first region) and the next thread's first region
-//     (a, b), by shuffle, shared memory, or global memory between blocks;
+//     rings before (R at its first region; with ring_jump.cuh's products the
+//     thread's own) and the next thread's first region (a, b), by shuffle,
+//     shared memory, or global memory between blocks;
 //   - region tables and radii in global memory, only in slices with beam
 //     particles to serve (stage 1 of RK4).
 // Crossed rings move to counted ranks (rank_sort.cuh) instead of through one
@@ -23,8 +24,8 @@
 // species (one thread took 53k of a slice's 183k cycles for 33 nodes: FP64
 // quotients one after the other) and kept in shared memory, and a ring beyond
 // a grid takes one FP64 quotient.
-// Measured on GB300, 24 wakes of 500-8000 rings in one launch: RK4 195 -> 96
-// us per slice, grids of 32 cells 103 -> 43.  Above 4 rings per thread the
+// Measured on GB300, 24 wakes of 500-8000 rings in one batch: RK4 190 -> 89
+// us per slice, grids of 32 cells 101 -> 40.  Above 4 rings per thread the
 // registers do not hold a thread's values (2 at 512 threads).
 #pragma once
 

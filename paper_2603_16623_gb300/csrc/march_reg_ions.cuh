@@ -11,7 +11,7 @@
 // only and travel with both species' t sums: nine barriers over the wake per
 // slice (the order vote, the two species' scans, own fields, t and matrices,
 // own d_zeta psi, Green's sums, regions, B^(p), the guard).
-// Measured on GB300, 24 wakes of 500-4000 cells in one launch: 62 -> 51 us
+// Measured on GB300, 24 wakes of 500-4000 cells in one batch: 62 -> 47 us
 // per slice (FP64, 8 wakes: 276 -> 233, its FP64 pipe's).
 #pragma once
 
